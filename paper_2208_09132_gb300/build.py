@@ -19,7 +19,7 @@ CSRC = os.path.join(PKG, "csrc")
 BUILD = os.path.join(PKG, "_build")
 LIBDIR = os.path.join(PKG, "lib")
 LIB = os.path.join(LIBDIR, "libcdugks.so")
-SOURCES = ["api.cu", "sweeps_f32.cu", "sweeps_f64.cu"]
+SOURCES = ["api.cu", "sweeps_f32.cu", "sweeps_f64.cu"] + [f"sweeps_f{p}_{d}.cu" for p in (32, 64) for d in (1, 2, 3)]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 
 

@@ -440,35 +440,38 @@ struct ShapeList<H, R...> {
     }
 };
 
-// The shapes of one precision for D = 1, 2, 3.
-template <typename T, typename L1, typename L2, typename L3>
-struct ShapeTable {
-    static int count(int D) { return D == 1 ? L1::count : (D == 2 ? L2::count : L3::count); }
-    static TileShape shape(int D, int id) { return D == 1 ? L1::shape(id) : (D == 2 ? L2::shape(id) : L3::shape(id)); }
-    static size_t smem(int D, int id) { return D == 1 ? L1::smem(id) : (D == 2 ? L2::smem(id) : L3::smem(id)); }
-    static int mode(int D, int id) { return D == 1 ? L1::mode(id) : (D == 2 ? L2::mode(id) : L3::mode(id)); }
-    static cudaError_t step(const Geo& g, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
-                            const void* phi_in) {
-        if (g.D == 1) return L1::template step<T>(g.tile_id, g, in, cur, s, ev, phi_in);
-        if (g.D == 2) return L2::template step<T>(g.tile_id, g, in, cur, s, ev, phi_in);
-        return L3::template step<T>(g.tile_id, g, in, cur, s, ev, phi_in);
-    }
-    static cudaError_t sweep_batch(int D, int id, bool B, const Item* it, int n, const Inst<T>* in, const int* cur,
-                                   cudaStream_t s) {
-        if (D == 1) return L1::template sweep_batch<T>(id, B, it, n, in, cur, s);
-        if (D == 2) return L2::template sweep_batch<T>(id, B, it, n, in, cur, s);
-        return L3::template sweep_batch<T>(id, B, it, n, in, cur, s);
-    }
-    static bool persistent(int D, int id) {
-        return D == 1 ? L1::persistent(id) : (D == 2 ? L2::persistent(id) : L3::persistent(id));
-    }
-    static cudaError_t persist(int D, int id, const PHead* h, const PItem* it, const Inst<T>* in, int* cur, PState* st,
-                               int n, int w, int th, cudaStream_t s) {
-        if (D == 1) return L1::template persist<T>(id, h, it, in, cur, st, n, w, th, s);
-        if (D == 2) return L2::template persist<T>(id, h, it, in, cur, st, n, w, th, s);
-        return L3::template persist<T>(id, h, it, in, cur, st, n, w, th, s);
-    }
+// The shapes of one precision and dimension as a table of functions: each
+// (precision, D) is instantiated in a translation unit of its own, so that the
+// build compiles them in parallel.
+template <typename T>
+struct ShapeOps {
+    int count;
+    TileShape (*shape)(int);
+    size_t (*smem)(int);
+    int (*mode)(int);
+    bool (*persistent)(int);
+    cudaError_t (*step)(int, const Geo&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*);
+    cudaError_t (*sweep_batch)(int, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t);
+    cudaError_t (*persist)(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t);
 };
+template <typename T, typename L>
+ShapeOps<T> ops_of() {
+    return {L::count, &L::shape, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
+            &L::template sweep_batch<T>, &L::template persist<T>};
+}
+const ShapeOps<float>& shapes_f32_1();
+const ShapeOps<float>& shapes_f32_2();
+const ShapeOps<float>& shapes_f32_3();
+const ShapeOps<double>& shapes_f64_1();
+const ShapeOps<double>& shapes_f64_2();
+const ShapeOps<double>& shapes_f64_3();
+template <typename T> const ShapeOps<T>& shapes_of(int D);
+template <> inline const ShapeOps<float>& shapes_of<float>(int D) {
+    return D == 1 ? shapes_f32_1() : (D == 2 ? shapes_f32_2() : shapes_f32_3());
+}
+template <> inline const ShapeOps<double>& shapes_of<double>(int D) {
+    return D == 1 ? shapes_f64_1() : (D == 2 ? shapes_f64_2() : shapes_f64_3());
+}
 
 template <typename T>
 cudaError_t launch_rawq_batch(int D, const QItem* items, int n, const Inst<T>* insts, const int* cur, cudaStream_t s) {
@@ -484,9 +487,10 @@ cudaError_t launch_rawq_batch(int D, const QItem* items, int n, const Inst<T>* i
 // tile shape, the raw face moments of the Shakhov members, the face
 // constants, sweep B per tile shape, the raw cell moments of the Shakhov
 // members, the W update.
-template <typename Table, typename T>
+template <typename T>
 cudaError_t run_batch_step(const BatchPlan& p, const Inst<T>* insts, int* cur, cudaStream_t s) {
     cudaError_t e;
+    const ShapeOps<T>& ops = shapes_of<T>(p.D);
     if (p.n_prep > 0) {
         switch (p.D) {
             case 1: e = launch_pdl(k_prep_batch<T, 1, true>, dim3(p.n_prep), dim3(kPrepCells), 0, s, p.prep_items, insts, cur); break;
@@ -496,7 +500,7 @@ cudaError_t run_batch_step(const BatchPlan& p, const Inst<T>* insts, int* cur, c
         if (e) return e;
     }
     for (int k = 0; k < p.ntile; ++k)
-        if ((e = Table::sweep_batch(p.D, p.tile_id[k], false, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
+        if ((e = ops.sweep_batch(p.tile_id[k], false, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
             return e;
     if ((e = launch_rawq_batch<T>(p.D, p.faceq_items, p.n_faceq, insts, cur, s))) return e;
     if (p.n_face > 0) {
@@ -508,7 +512,7 @@ cudaError_t run_batch_step(const BatchPlan& p, const Inst<T>* insts, int* cur, c
         if (e) return e;
     }
     for (int k = 0; k < p.ntile; ++k)
-        if ((e = Table::sweep_batch(p.D, p.tile_id[k], true, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
+        if ((e = ops.sweep_batch(p.tile_id[k], true, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
             return e;
     if ((e = launch_rawq_batch<T>(p.D, p.cellq_items, p.n_cellq, insts, cur, s))) return e;
     if (p.n_cell > 0) {
