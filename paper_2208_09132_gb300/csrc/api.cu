@@ -16,6 +16,7 @@
 #include "../../include/cdugks.h"
 #include "launch.cuh"
 #include "persist.cuh"
+#include "bflux.cuh"
 
 using cdg::BatchPlan;
 using cdg::Bufs;
@@ -48,7 +49,7 @@ constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
 struct Layout {
-    size_t phi[2], pb, sg, fv[3], W, cellc, cellc0, facec[3], wf[3], mf[3], vel, refl, io, status, inst;
+    size_t phi[2], pb, sg, fv[3], W, cellc, cellc0, facec[3], wf[3], mf[3], vel, refl, vint, vrec, slots, cint, crec, io, status, inst;
     size_t hq, qs, qf[3];     // Shakhov model only
     size_t force;             // acceleration only
     size_t xc, xc0, xf[3];    // lean shapes only: separable factor tables
@@ -56,9 +57,11 @@ struct Layout {
 };
 
 // Optional workspace buffers, by the sweep modes that need them.
-enum { BUF_PHIBAR = 1, BUF_SLOPES = 2, BUF_FACES = 4, BUF_FORCE = 8, BUF_XTAB = 16 };
+enum { BUF_PHIBAR = 1, BUF_SLOPES = 2, BUF_FACES = 4, BUF_FORCE = 8, BUF_XTAB = 16, BUF_VISITS = 32, BUF_CHUNKS = 64 };
 int buffers_of(int mode) {
     int b = 0;
+    if (cdg::mode_upwind(mode)) b |= BUF_VISITS;
+    if (cdg::mode_faces(mode) && !cdg::mode_acc(mode)) b |= BUF_CHUNKS;
     if (cdg::mode_lean(mode)) b |= BUF_XTAB;
     if (cdg::mode_acc(mode)) b |= BUF_FORCE;
     if (cdg::mode_source(mode) != cdg::MODE_FUSED) b |= BUF_PHIBAR;
@@ -94,6 +97,13 @@ struct cdugks {
     std::vector<double> vel;  // [Nvp][8]: xi_0, xi_1, xi_2, w, |xi|^2/2, 0, 0, 0
     std::vector<float> vel32; // the same table rounded to float (FP32 storage)
     std::vector<int> refl;    // [8][Nvp]
+    std::vector<int> vint;    // visits of sweep A (Bufs::vint, Bufs::vrec)
+    std::vector<double> vrec;
+    std::vector<float> vrec32;
+    std::vector<int> cint;    // chunk records of sweep B (Bufs::cint, Bufs::crec)
+    std::vector<double> crec;
+    std::vector<float> crec32;
+    std::vector<int> slots;   // [gcap][3][2] (Bufs::slots)
     // captured steps (cdugks_capture): one graph per parity of the state buffer it starts from
     cudaGraph_t graph[2] = {nullptr, nullptr};
     cudaGraphExec_t gexec[2] = {nullptr, nullptr};
@@ -149,10 +159,132 @@ int groups_for(const cdugks* h, int requested) {
     return (int)G;
 }
 
+// The visits of sweep A with upwind owners (usweep.cuh), sorted by their sides
+// and mixed axes, then (velocity rows of whole chunks) with the axis-0 chunk
+// varying slowest and axis 1 fastest, so that a place's axis-0 factors stay the
+// same over long runs; and the chunks in that last order for sweep B.  Padding
+// and nodes at xi_a = 0 are stored as negative; such a node is summed half on
+// either side.
+void build_visits(cdugks* h) {
+    const Geo& g = h->g;
+    const int D = g.D, DM = cdg::mixed_axes(D), mask = ((1 << D) - 1) & ~((1 << DM) - 1);   // axes with visits of their own
+    std::vector<unsigned char> pos(g.Nvp, 0), zero(g.Nvp, 0);      // bits per axis: xi_a > 0; xi_a = 0
+    for (int i = 0; i < g.Nvp; ++i)
+        for (int a = 0; a < D; ++a) {
+            const double x = i < h->Nv ? h->vel[(size_t)i * 8 + a] : 0.0;
+            pos[i] |= (unsigned char)((x > 0.0 ? 1 : 0) << a);
+            zero[i] |= (unsigned char)((x == 0.0 ? 1 : 0) << a);
+        }
+    struct Visit {
+        int key, vt, flags, own;       // own: the signs of its axes in mask
+    };
+    const int n0c = g.nv1[0] / VC, m = g.nv1[1] * g.nv1[2];
+    auto order = [&](int vt) { return g.xal ? (vt % n0c) * m + vt / n0c : vt; };
+    std::vector<Visit> vis, chunks;
+    vis.reserve(g.NVT + 16);
+    chunks.resize(g.NVT);
+    for (int vt = 0; vt < g.NVT; ++vt) {
+        const unsigned char* ps = &pos[(size_t)vt * VC];
+        const unsigned char* zs = &zero[(size_t)vt * VC];
+        chunks[order(vt)] = Visit{0, vt, 0, 0};
+        unsigned seen = 0;
+        for (int v = 0; v < VC; ++v) {
+            const int own = ps[v] & mask;
+            if ((seen >> own) & 1) continue;
+            seen |= 1u << own;
+            unsigned flags = 0;
+            for (int a = 0; a < D; ++a) {
+                unsigned plus = 0, minus = 0;
+                bool z = false;
+                for (int w = 0; w < VC; ++w) {
+                    if ((ps[w] & mask) != own) continue;
+                    ((ps[w] >> a) & 1 ? plus : minus) |= 1u << w;
+                    z = z || (((zs[w] >> a) & 1) && vt * VC + w < h->Nv);
+                }
+                const bool both = a < DM && ((plus && minus) || z);
+                if (both) flags |= 9u << a | plus << (8 + 4 * a) | minus << (20 + 4 * a);
+                else flags |= (plus ? 1u << a | plus << (8 + 4 * a) : minus << (8 + 4 * a));
+            }
+            vis.push_back(Visit{order(vt), vt, (int)flags, own});
+        }
+    }
+    std::stable_sort(vis.begin(), vis.end(), [](const Visit& x, const Visit& y) {
+        const int cx = cdg::visit_class(x.flags), cy = cdg::visit_class(y.flags);
+        return cx != cy ? cx < cy : x.key < y.key;
+    });
+    h->g.nvis = (int)vis.size();
+    h->g.mixed = std::any_of(vis.begin(), vis.end(), [](const Visit& v) { return (cdg::visit_class(v.flags) & 56) != 0; });
+    // the records' values go to the storage precision's table only
+    auto records = [&](const std::vector<Visit>& list, int ni, int nv, std::vector<int>& ints, auto& vals) {
+        using V = typename std::decay<decltype(vals[0])>::type;
+        ints.assign((size_t)ni * list.size(), 0);
+        vals.assign((size_t)nv * VC * list.size(), V(0));
+        for (size_t j = 0; j < list.size(); ++j) {
+            int* vi = &ints[(size_t)ni * j];
+            V* vr = &vals[(size_t)nv * VC * j];
+            const Visit& vs = list[j];
+            vi[0] = vs.vt;
+            vi[1] = vs.flags;
+            for (int v = 0; v < VC; ++v) {
+                const int i = vs.vt * VC + v;
+                const double* rec = &h->vel[(size_t)i * 8];
+                for (int a = 0; a < 3; ++a) {
+                    vr[a * VC + v] = (V)rec[a];
+                    vr[(4 + a) * VC + v] = (V)-rec[5 + a];
+                }
+                vr[3 * VC + v] = (V)rec[4];
+                if (nv == cdg::kChunkVecs) vr[7 * VC + v] = (V)rec[3];
+                else if ((pos[i] & mask) == vs.own)
+                    for (int a = 0; a < D; ++a) {
+                        const bool z = (zero[i] >> a) & 1, plus = (pos[i] >> a) & 1;
+                        const double w = z ? 0.5 * rec[3] : rec[3];
+                        if (z) vi[16] |= 1 << (4 * a + v);
+                        if (!cdg::visit_mixed(vs.flags, a)) vr[(7 + a) * VC + v] = (V)w;
+                        else {
+                            if (plus || z) vr[(7 + a) * VC + v] = (V)w;
+                            if (!plus) vr[(10 + a) * VC + v] = (V)w;
+                        }
+                    }
+                const bool pad = i >= h->Nv;
+                vi[4 + v] = pad ? -1 : i % g.nv1[0];
+                vi[8 + v] = pad ? 0 : g.xrow[1] + (i / g.nv1[0]) % g.nv1[1];
+                vi[12 + v] = pad ? 0 : g.xrow[2] + i / (g.nv1[0] * g.nv1[1]);
+            }
+            vi[2] = vi[8];
+            vi[3] = vi[12];
+        }
+    };
+    if (h->prec == CDUGKS_FP32) {
+        records(vis, cdg::kVisitInts, cdg::kVisitVecs, h->vint, h->vrec32);
+        records(chunks, cdg::kChunkInts, cdg::kChunkVecs, h->cint, h->crec32);
+    } else {
+        records(vis, cdg::kVisitInts, cdg::kVisitVecs, h->vint, h->vrec);
+        records(chunks, cdg::kChunkInts, cdg::kChunkVecs, h->cint, h->crec);
+    }
+}
+
+// The velocity groups, and the slots of the face-W partial sums: one per group
+// and sign among its visits where sweep A sums one side of a face at a time,
+// else one per group.
 void set_groups(cdugks* h, int G) {
     Geo& g = h->g;
     g.ntpg = (g.NVT + G - 1) / G;
     g.G = (g.NVT + g.ntpg - 1) / g.ntpg;
+    for (int a = 0; a < 3; ++a) g.ws[a] = g.G;
+    const int mode = tile_mode(h->prec, g.D, g.tile_id);
+    g.upw = cdg::mode_upwind(mode) && !(cdg::mode_sk(mode) && h->zero_node);
+    if (!g.upw) return;
+    h->slots.assign((size_t)g.G * 6, -1);
+    for (int a = 0; a < 3; ++a) g.ws[a] = 0;
+    for (int gr = 0; gr < g.G; ++gr)
+        for (int a = 0; a < g.D; ++a)
+            for (int side = 0; side < 2; ++side) {
+                bool has = false;
+                for (long long j = (long long)gr * g.nvis / g.G; j < (long long)(gr + 1) * g.nvis / g.G && !has; ++j)
+                    has = cdg::visit_plus(h->vint[cdg::kVisitInts * (size_t)j + 1], a) == side ||
+                          (!side && cdg::visit_mixed(h->vint[cdg::kVisitInts * (size_t)j + 1], a));
+                if (has) h->slots[(size_t)(gr * 3 + a) * 2 + side] = g.ws[a]++;
+            }
 }
 
 void make_layout(cdugks* h) {
@@ -179,11 +311,18 @@ void make_layout(cdugks* h) {
     for (int a = 0; a < 3; ++a) {
         const long long nf = a < g.D ? g.nf[a] : 0;
         L.facec[a] = take(h->facec_bytes * nf);
-        L.wf[a] = take(sizeof(double) * (size_t)h->gcap * NM * nf);
+        L.wf[a] = take(sizeof(double) * (size_t)h->gcap * ((h->bufs_cap & BUF_VISITS) ? 2 : 1) * NM * nf);
         L.mf[a] = take(sizeof(double) * (size_t)h->gcap * NM * nf);
     }
     L.vel = take(h->elt * 8 * g.Nvp);
     L.refl = take(sizeof(int) * 8 * g.Nvp);
+    const bool vis = (h->bufs_cap & BUF_VISITS) != 0;
+    L.vint = vis ? take(sizeof(int) * h->vint.size()) : 0;
+    L.vrec = vis ? take(h->elt * std::max(h->vrec.size(), h->vrec32.size())) : 0;
+    L.slots = vis ? take(sizeof(int) * 6 * (size_t)h->gcap) : 0;
+    const bool chk = (h->bufs_cap & BUF_CHUNKS) != 0;
+    L.cint = chk ? take(sizeof(int) * h->cint.size()) : 0;
+    L.crec = chk ? take(h->elt * std::max(h->crec.size(), h->crec32.size())) : 0;
     L.io = take(sizeof(double) * std::max(NM, g.D * g.D + g.D) * g.Nc);   // moments, or P and q
     const bool sk = h->collision == CDUGKS_COLLISION_SHAKHOV;
     const int NQ = g.D + g.D * (g.D + 1) / 2;
@@ -221,6 +360,13 @@ Bufs<T> bufs(const cdugks* h, int in) {
     }
     b.vel = reinterpret_cast<const T*>(p + L.vel);
     b.refl = reinterpret_cast<const int*>(p + L.refl);
+    const bool vis = (h->bufs_cap & BUF_VISITS) != 0;
+    b.vint = vis ? reinterpret_cast<const int*>(p + L.vint) : nullptr;
+    b.vrec = vis ? reinterpret_cast<const T*>(p + L.vrec) : nullptr;
+    b.slots = vis ? reinterpret_cast<const int*>(p + L.slots) : nullptr;
+    const bool chk = (h->bufs_cap & BUF_CHUNKS) != 0;
+    b.cint = chk ? reinterpret_cast<const int*>(p + L.cint) : nullptr;
+    b.crec = chk ? reinterpret_cast<const T*>(p + L.crec) : nullptr;
     b.status = reinterpret_cast<int*>(p + L.status);
     const bool sk = h->collision == CDUGKS_COLLISION_SHAKHOV;
     b.hq = sk ? reinterpret_cast<double*>(p + L.hq) : nullptr;
@@ -261,9 +407,14 @@ Inst<T> inst_of(const cdugks* h) {
     return in;
 }
 
-// The instance record every kernel of this handle reads (geometry + buffers).
+// The instance record every kernel of this handle reads (geometry + buffers),
+// and the slots of its velocity groups.
 int upload_inst(cdugks* h) {
     cudaError_t e;
+    if (h->g.upw &&
+        (e = cudaMemcpyAsync(h->base + h->lay.slots, h->slots.data(), sizeof(int) * h->slots.size(),
+                             cudaMemcpyHostToDevice, h->stream)))
+        return cuda_fail(e, "upload group slots");
     if (h->prec == CDUGKS_FP32) {
         const Inst<float> in = inst_of<float>(h);
         e = cudaMemcpyAsync(h->base + h->lay.inst, &in, sizeof(in), cudaMemcpyHostToDevice, h->stream);
@@ -448,6 +599,10 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     g.Pr = phys->Pr;
     // with Pr = 1 the TEDDF b-source coefficient (Pr - 1)/tau vanishes exactly
     g.nosrc = phys->Pr == 1.0;
+    g.mirror = 1;
+    for (int a = 0; a < D; ++a)
+        for (int s = 0; s < 2; ++s) g.mirror = g.mirror && g.bc[a][s] != CDUGKS_BC_DIRICHLET;
+    build_visits(h);
     set_tiles(h, 0);
     h->vel32 = cast_vec<float>(h->vel);
     h->gsel = 0;
@@ -656,6 +811,24 @@ int cdugks_bind(cdugks_t* h, void* device_ptr, size_t bytes, void* cuda_stream) 
     if ((e = cudaMemcpyAsync(h->base + h->lay.refl, h->refl.data(), h->refl.size() * sizeof(int),
                              cudaMemcpyHostToDevice, h->stream)))
         return cuda_fail(e, "upload reflection table");
+    if (h->bufs_cap & BUF_VISITS) {
+        const void* vr = h->prec == CDUGKS_FP32 ? static_cast<const void*>(h->vrec32.data())
+                                                : static_cast<const void*>(h->vrec.data());
+        if ((e = cudaMemcpyAsync(h->base + h->lay.vint, h->vint.data(), sizeof(int) * h->vint.size(),
+                                 cudaMemcpyHostToDevice, h->stream)) ||
+            (e = cudaMemcpyAsync(h->base + h->lay.vrec, vr, h->elt * std::max(h->vrec.size(), h->vrec32.size()),
+                                 cudaMemcpyHostToDevice, h->stream)))
+            return cuda_fail(e, "upload visits");
+    }
+    if (h->bufs_cap & BUF_CHUNKS) {
+        const void* cr = h->prec == CDUGKS_FP32 ? static_cast<const void*>(h->crec32.data())
+                                                : static_cast<const void*>(h->crec.data());
+        if ((e = cudaMemcpyAsync(h->base + h->lay.cint, h->cint.data(), sizeof(int) * h->cint.size(),
+                                 cudaMemcpyHostToDevice, h->stream)) ||
+            (e = cudaMemcpyAsync(h->base + h->lay.crec, cr, h->elt * std::max(h->crec.size(), h->crec32.size()),
+                                 cudaMemcpyHostToDevice, h->stream)))
+            return cuda_fail(e, "upload chunk records");
+    }
     if ((e = cudaMemsetAsync(h->base + h->lay.status, 0, 256, h->stream))) return cuda_fail(e, "clear status");
     if ((e = cudaStreamSynchronize(h->stream))) return cuda_fail(e, "cudaStreamSynchronize");
     (void)g;
@@ -695,8 +868,8 @@ int cdugks_init(cdugks_t* h, const double* rho_u_T) {
 namespace {
 cudaError_t launch_one_step(cdugks* h) {
     const void* phi_in = h->base + h->lay.phi[h->cur];
-    if (h->prec == CDUGKS_FP32) return cdg::launch_step_f32(h->g, dinst<float>(h), h->cur, h->stream, nullptr, phi_in);
-    return cdg::launch_step_f64(h->g, dinst<double>(h), h->cur, h->stream, nullptr, phi_in);
+    if (h->prec == CDUGKS_FP32) return cdg::launch_step_f32(h->g, bufs<float>(h, h->cur), dinst<float>(h), h->cur, h->stream, nullptr, phi_in);
+    return cdg::launch_step_f64(h->g, bufs<double>(h, h->cur), dinst<double>(h), h->cur, h->stream, nullptr, phi_in);
 }
 }  // namespace
 
@@ -766,8 +939,8 @@ int cdugks_profile_step(cdugks_t* h, int nsteps, double* ms_out) {
     for (int s = 0; s < nsteps && e == cudaSuccess; ++s) {
         cudaEvent_t* es = &ev[(size_t)s * 5];
         const void* phi_in = h->base + h->lay.phi[h->cur];
-        if (h->prec == CDUGKS_FP32) e = cdg::launch_step_f32(h->g, dinst<float>(h), h->cur, h->stream, es, phi_in);
-        else e = cdg::launch_step_f64(h->g, dinst<double>(h), h->cur, h->stream, es, phi_in);
+        if (h->prec == CDUGKS_FP32) e = cdg::launch_step_f32(h->g, bufs<float>(h, h->cur), dinst<float>(h), h->cur, h->stream, es, phi_in);
+        else e = cdg::launch_step_f64(h->g, bufs<double>(h, h->cur), dinst<double>(h), h->cur, h->stream, es, phi_in);
         if (e) break;
         h->cur = 1 - h->cur;
         h->steps += 1;
@@ -1039,13 +1212,14 @@ struct cdugks_batch {
     std::vector<cdugks*> mem;
     int prec, D;
     std::vector<int> tile_ids;                 // distinct tile shapes, in plan order
-    std::vector<std::vector<Item>> sweep_items;
+    std::vector<int> list_keys;                // sweep lists: 2 tile id + (sweep A with upwind owners)
+    std::vector<std::vector<Item>> sweep_items, sweep_b_items;
     std::vector<RItem> face_items, cell_items;
     std::vector<RItem> prep_items;             // acceleration members: the pre-pass
     std::vector<QItem> faceq_items, cellq_items;   // Shakhov members: raw moments
     std::vector<unsigned char> insts;          // host image of the Inst<T> table
     std::vector<int> cur;
-    size_t off_insts, off_cur, off_sweep[cdg::kMaxBatchShapes], off_face, off_cell, total;
+    size_t off_insts, off_cur, off_sweep[cdg::kMaxBatchLists], off_sweep_b[cdg::kMaxBatchLists], off_face, off_cell, total;
     size_t off_prep, off_faceq, off_cellq;
     unsigned char* base;
     cudaStream_t stream;
@@ -1081,11 +1255,14 @@ BatchPlan plan_of(const cdugks_batch* b) {
     BatchPlan p;
     std::memset(&p, 0, sizeof(p));
     p.D = b->D;
-    p.ntile = (int)b->tile_ids.size();
+    p.ntile = (int)b->list_keys.size();
     for (int k = 0; k < p.ntile; ++k) {
-        p.tile_id[k] = b->tile_ids[k];
+        p.tile_id[k] = b->list_keys[k] / 2;
+        p.upw[k] = b->list_keys[k] % 2 != 0;
         p.sweep_items[k] = reinterpret_cast<const Item*>(b->base + b->off_sweep[k]);
         p.n_sweep[k] = (int)b->sweep_items[k].size();
+        p.sweep_b_items[k] = reinterpret_cast<const Item*>(b->base + b->off_sweep_b[k]);
+        p.n_sweep_b[k] = (int)b->sweep_b_items[k].size();
     }
     p.face_items = reinterpret_cast<const RItem*>(b->base + b->off_face);
     p.n_face = (int)b->face_items.size();
@@ -1177,21 +1354,35 @@ int batch_plan(cdugks_batch* b) {
     std::sort(b->tile_ids.begin(), b->tile_ids.end());
     if (b->tile_ids.size() > (size_t)cdg::kMaxBatchShapes)     // before any per-shape table is filled
         return fail(CDUGKS_ERR_INVALID, "too many tile shapes in one batch");
-    b->sweep_items.assign(b->tile_ids.size(), {});
+    b->list_keys.clear();
+    for (int i = 0; i < n; ++i) {
+        const int key = 2 * b->mem[i]->g.tile_id + (b->mem[i]->g.upw ? 1 : 0);
+        if (std::find(b->list_keys.begin(), b->list_keys.end(), key) == b->list_keys.end()) b->list_keys.push_back(key);
+    }
+    std::sort(b->list_keys.begin(), b->list_keys.end());
+    b->sweep_items.assign(b->list_keys.size(), {});
+    b->sweep_b_items.assign(b->list_keys.size(), {});
     for (int i = 0; i < n; ++i) {
         const Geo& g = b->mem[i]->g;
-        const int k = (int)(std::find(b->tile_ids.begin(), b->tile_ids.end(), g.tile_id) - b->tile_ids.begin());
+        const int key = 2 * g.tile_id + (g.upw ? 1 : 0);
+        const int k = (int)(std::find(b->list_keys.begin(), b->list_keys.end(), key) - b->list_keys.begin());
         const int tiles = g.tiles[0] * g.tiles[1] * g.tiles[2];
         for (int t = 0; t < tiles; ++t)
             for (int gr = 0; gr < g.G; ++gr) b->sweep_items[k].push_back(Item{i, t, gr, 0});
+        const cdg::TileShape bs = b->prec == CDUGKS_FP32 ? cdg::b_tile_shape_f32(D, g.tile_id) : cdg::b_tile_shape_f64(D, g.tile_id);
+        int btiles = 1;
+        for (int a = 0; a < D; ++a) btiles *= (g.n[a] + bs.t[a] - 1) / bs.t[a];
+        for (int t = 0; t < btiles; ++t)
+            for (int gr = 0; gr < g.G; ++gr) b->sweep_b_items[k].push_back(Item{i, t, gr, 0});
     }
-    for (auto& v : b->sweep_items)
-        std::stable_sort(v.begin(), v.end(), [&](const Item& x, const Item& y) {
-            const Geo& gx = b->mem[x.inst]->g;
-            const Geo& gy = b->mem[y.inst]->g;
-            const int wx = std::min(gx.ntpg, gx.NVT - x.grp * gx.ntpg), wy = std::min(gy.ntpg, gy.NVT - y.grp * gy.ntpg);
-            return wx > wy;
-        });
+    for (auto* lists : {&b->sweep_items, &b->sweep_b_items})
+        for (auto& v : *lists)
+            std::stable_sort(v.begin(), v.end(), [&](const Item& x, const Item& y) {
+                const Geo& gx = b->mem[x.inst]->g;
+                const Geo& gy = b->mem[y.inst]->g;
+                const int wx = std::min(gx.ntpg, gx.NVT - x.grp * gx.ntpg), wy = std::min(gy.ntpg, gy.NVT - y.grp * gy.ntpg);
+                return wx > wy;
+            });
     // face and cell ranges: whole blocks of the kernel that runs them (64 threads,
     // or the persistent shape's threads), sized so that the batch has about 2048
     // of each (a few ranges of a lone member would leave most SMs idle while
@@ -1296,7 +1487,10 @@ int batch_plan(cdugks_batch* b) {
     }
     b->off_insts = take(b->insts.size());
     b->off_cur = take(sizeof(int) * n);
-    for (size_t k = 0; k < b->sweep_items.size(); ++k) b->off_sweep[k] = take(sizeof(Item) * b->sweep_items[k].size());
+    for (size_t k = 0; k < b->sweep_items.size(); ++k) {
+        b->off_sweep[k] = take(sizeof(Item) * b->sweep_items[k].size());
+        b->off_sweep_b[k] = take(sizeof(Item) * b->sweep_b_items[k].size());
+    }
     b->off_face = take(sizeof(RItem) * b->face_items.size());
     b->off_cell = take(sizeof(RItem) * b->cell_items.size());
     b->off_prep = take(sizeof(RItem) * b->prep_items.size());
@@ -1435,7 +1629,9 @@ int cdugks_batch_bind(cdugks_batch_t* b, void* device_ptr, size_t bytes, void* c
         return cuda_fail(e, "upload batch tables");
     for (size_t k = 0; k < b->sweep_items.size() && !b->pers; ++k)
         if ((e = cudaMemcpyAsync(b->base + b->off_sweep[k], b->sweep_items[k].data(),
-                                 sizeof(Item) * b->sweep_items[k].size(), cudaMemcpyHostToDevice, b->stream)))
+                                 sizeof(Item) * b->sweep_items[k].size(), cudaMemcpyHostToDevice, b->stream)) ||
+            (e = cudaMemcpyAsync(b->base + b->off_sweep_b[k], b->sweep_b_items[k].data(),
+                                 sizeof(Item) * b->sweep_b_items[k].size(), cudaMemcpyHostToDevice, b->stream)))
             return cuda_fail(e, "upload sweep items");
     if (!b->pers &&
         ((e = cudaMemcpyAsync(b->base + b->off_face, b->face_items.data(), sizeof(RItem) * b->face_items.size(),
@@ -1655,6 +1851,7 @@ int noalloc_run(cdugks* h, const void* phi_in, void* phi_out, double* W, cudaStr
     for (int G = std::max(1, g.G);; G = std::max(1, G / 2)) {
         g.ntpg = (g.NVT + G - 1) / G;
         g.G = (g.NVT + g.ntpg - 1) / g.ntpg;
+        for (int a = 0; a < 3; ++a) g.ws[a] = g.G;
         size_t off = 0;
         auto take = [&](size_t bytes) {
             const size_t o = off;
@@ -1718,10 +1915,10 @@ int noalloc_run(cdugks* h, const void* phi_in, void* phi_out, double* W, cudaStr
     const Inst<T>* din = reinterpret_cast<const Inst<T>*>(base + off_inst);
     if constexpr (std::is_same<T, float>::value) {
         e = cdg::launch_cellc_f32(g, din, 0, st);
-        if (!e) e = cdg::launch_step_f32(g, din, 0, st);
+        if (!e) e = cdg::launch_step_f32(g, b, din, 0, st);
     } else {
         e = cdg::launch_cellc_f64(g, din, 0, st);
-        if (!e) e = cdg::launch_step_f64(g, din, 0, st);
+        if (!e) e = cdg::launch_step_f64(g, b, din, 0, st);
     }
     if (e) return cuda_fail(e, "allocation-free step launch");
     // (copies from pageable host memory return once the source has been staged,

@@ -94,7 +94,15 @@ struct Geo {
     int xrow[3];
     int xrows;
     int xal;          // nv1_0 is a multiple of VC: a chunk's four velocities share their other indices
+    // Sweep A with upwind owners (usweep.cuh):
+    int upw;          // this instance's sweep A is usweep.cuh's
+    int mixed;        // some visit is mixed along an axis
+    int nvis;         // visits (chunk, sign pattern), in the order of Bufs::vint
+    int mirror;       // no Dirichlet end: ghosts are images of cells with all their neighbours
+    int ws[3];        // partial sums of the face W per axis: the group slots of sweep A (G where it sums both sides)
 };
+
+constexpr int kVisitInts = 20, kVisitVecs = 13, kChunkInts = 16, kChunkVecs = 8;
 
 template <typename T> struct CellC;
 template <typename T> struct FaceC;
@@ -110,11 +118,20 @@ struct Bufs {
     CellC<T>* cellc;      // [Nc] constants of W^n (written by the W update / init)
     CellC<T>* cellc0;     // [Nc] constants of W^0 (Dirichlet ghosts)
     FaceC<T>* facec[3];   // [nf_a] constants of the face W (between the sweeps)
-    double* wf[3];        // [G][2+D][nf_a] face W partial sums (sweep A)
+    double* wf[3];        // [ws_a][2+D][nf_a] face W partial sums (sweep A)
     double* mf[3];        // [G][2+D][nf_a] face flux-moment partial sums (sweep B)
     const T* vel;         // [Nvp][8] per velocity: xi_0, xi_1, xi_2, w, |xi|^2/2, 2h xi_0/dx_0, 2h xi_1/dx_1,
                           // 2h xi_2/dx_2 (w = 0 on padding)
     const int* refl;      // [8][Nvp] velocity index with the components of mask reversed
+    // visits of sweep A with upwind owners: per visit kVisitInts ints (chunk, flags, axis-1 and axis-2 row of its
+    // first lane, the rows per lane of axes 0 (-1 padding), 1, 2, the lanes at xi_a = 0) and kVisitVecs chunk-wide
+    // values (xi_0..2, |xi|^2/2, -2h xi_a/dx_a, the weights per axis of the main side, of the other side); per
+    // group and axis the wf slot of either side (-1 none)
+    const int* vint;
+    const T* vrec;
+    const int* slots;     // [G][3][right cells' side, left cells' side]
+    const int* cint;      // per chunk kChunkInts ints (as above) and kChunkVecs values (up to the weights), for sweep B
+    const T* crec;
     int* status;
     // Shakhov model only (null otherwise); NQ = D + D(D+1)/2 raw moments
     double* hq;           // [D][Nc] heat flux of the current time level, tracked like W
@@ -167,9 +184,16 @@ template <> struct Num<float> {
     static __host__ __device__ __forceinline__ float irt_scale() { return -1.3862943611198906f; }
     // half the van Leer slope: s1 s2 / (s1 + s2) (the factor 2 is folded into the
     // reconstruction coefficients)
+    static __device__ __forceinline__ float rcp(float x) {
+        float y;   // hardware reciprocal (1 ulp; subnormal inputs and results flushed)
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+        return y;
+    }
+    // The quotient as p rcp(s): p > 0 implies |s| > 2^-74, so the flushing form
+    // of the reciprocal loses nothing there.
     static __device__ __forceinline__ float vanleer(float s1, float s2) {
-        float p = s1 * s2;
-        return p > 0.f ? __fdividef(p, s1 + s2) : 0.f;
+        const float p = s1 * s2;
+        return p > 0.f ? p * rcp(s1 + s2) : 0.f;
     }
 };
 template <> struct Num<double> {
@@ -800,6 +824,13 @@ __host__ __device__ constexpr bool mode_nosrc(int mode) { return (mode & (MODE_N
 __host__ __device__ constexpr int mode_halo(int mode) { return mode_r2(mode) ? 3 : 2; }
 __host__ __device__ constexpr bool mode_lean(int mode) { return (mode & MODE_LEAN) != 0; }
 __host__ __device__ constexpr bool mode_xf(int mode) { return (mode & MODE_XF) != 0; }
+// Shapes whose sweep A is usweep.cuh's: the lean shapes and the fused
+// face-store shapes of the upwind-cell reconstruction, of either collision
+// model (the Shakhov model on velocity grids with a node at 0 keeps the fused
+// sweep: its heat flux reads the stored face values of those nodes, Geo::upw).
+__host__ __device__ constexpr bool mode_upwind(int mode) {
+    return mode_faces(mode) && mode_source(mode) == MODE_FUSED && !mode_r2(mode) && !mode_acc(mode);
+}
 
 template <typename T, int D, int T0, int T1, int T2, int MODE = MODE_FUSED>
 struct Smem {
@@ -2535,7 +2566,7 @@ __device__ __forceinline__ void facec_body(const Geo& g, const Bufs<T>& bf, int 
     double W[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
     {
         double s[NM];
-        group_sums<NM>(bf.wf[a] + f, (size_t)g.nf[a], g.G, s);
+        group_sums<NM>(bf.wf[a] + f, (size_t)g.nf[a], g.ws[a], s);
         for (int m = 0; m < NM; ++m) W[m] = s[m];
     }
     if (g.accel) {   // eqs. rhoubar, rhoEbar: + (h/2) rho a, then + (h/2) (rho u) . a

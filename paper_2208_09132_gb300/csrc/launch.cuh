@@ -13,13 +13,17 @@ struct TileShape {
 };
 
 // Work of one batched step: sweep items grouped by tile shape, face and cell ranges.
-constexpr int kMaxBatchShapes = 8;
+// A shape whose members take different sweeps A (Geo::upw) has a list for each.
+constexpr int kMaxBatchShapes = 8, kMaxBatchLists = 2 * kMaxBatchShapes;
 struct BatchPlan {
     int D;
-    int ntile;
-    int tile_id[kMaxBatchShapes];
-    const Item* sweep_items[kMaxBatchShapes];
-    int n_sweep[kMaxBatchShapes];
+    int ntile;                   // lists
+    int tile_id[kMaxBatchLists];
+    bool upw[kMaxBatchLists];
+    const Item* sweep_items[kMaxBatchLists];
+    int n_sweep[kMaxBatchLists];
+    const Item* sweep_b_items[kMaxBatchLists];   // sweep B has its own tiles
+    int n_sweep_b[kMaxBatchLists];
     const RItem* face_items;
     int n_face;
     const RItem* cell_items;
@@ -37,6 +41,8 @@ int tile_count_f32(int D);
 int tile_count_f64(int D);
 TileShape tile_shape_f32(int D, int id);
 TileShape tile_shape_f64(int D, int id);
+TileShape b_tile_shape_f32(int D, int id);      // of sweep B's batched items
+TileShape b_tile_shape_f64(int D, int id);
 size_t sweep_smem_f32(int D, int id);
 size_t sweep_smem_f64(int D, int id);
 // Sweep mode of a shape (MODE_FUSED / MODE_PREP / MODE_STORED): prepared and
@@ -48,12 +54,13 @@ int tile_mode_f64(int D, int id);
 // and use orientation `cur` (read state buffer cur, write the other).
 // One time step: sweep A, face constants, sweep B, W update (+ cell constants of W^{n+1}).
 // ev: null, or five events recorded before, between and after the four phases.
-// phi_in: the device address of the state buffer the step reads (the tensor
+// hb: the buffers of orientation cur (sweep A with upwind owners takes them as a
+// kernel parameter).  phi_in: the device address of the state buffer the step reads (the tensor
 // maps of sweep A's TMA staging), or null (per-cell staging only).
-cudaError_t launch_step_f32(const Geo& g, const Inst<float>* in, int cur, cudaStream_t s, cudaEvent_t* ev = nullptr,
-                            const void* phi_in = nullptr);
-cudaError_t launch_step_f64(const Geo& g, const Inst<double>* in, int cur, cudaStream_t s, cudaEvent_t* ev = nullptr,
-                            const void* phi_in = nullptr);
+cudaError_t launch_step_f32(const Geo& g, const Bufs<float>& hb, const Inst<float>* in, int cur, cudaStream_t s,
+                            cudaEvent_t* ev = nullptr, const void* phi_in = nullptr);
+cudaError_t launch_step_f64(const Geo& g, const Bufs<double>& hb, const Inst<double>* in, int cur, cudaStream_t s,
+                            cudaEvent_t* ev = nullptr, const void* phi_in = nullptr);
 // One time step of every instance of a batch.
 cudaError_t launch_batch_step_f32(const BatchPlan& p, const Inst<float>* insts, int* cur, cudaStream_t s);
 cudaError_t launch_batch_step_f64(const BatchPlan& p, const Inst<double>* insts, int* cur, cudaStream_t s);

@@ -23,6 +23,7 @@
 #pragma once
 
 #include "kernels.cuh"
+#include "bflux.cuh"
 
 namespace cdg {
 
@@ -59,12 +60,12 @@ __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
 
 template <typename T, int D, int TX, int TY, int TZ, int MODE>
 struct PersistSmem {
-    static constexpr bool FACES = mode_faces(MODE);
-    static constexpr size_t a = Smem<T, D, TX, TY, TZ, MODE>::bytes(false);
-    static constexpr size_t b = FACES ? FluxSmem<T, D, TX, TY, TZ>::bytes : Smem<T, D, TX, TY, TZ, MODE>::bytes(true);
+    static_assert(mode_upwind(MODE), "the persistent shapes are fused face-store shapes");
+    static constexpr size_t a = USmem<T, D, TX, TY, TZ, false>::bytes;
+    static constexpr size_t b = BSmem<T, D, TX, TY, TZ, false, false>::bytes;
     static constexpr size_t bytes = a > b ? a : b;
-    static constexpr int occ_a = Occ<T, D, TX, TY, TZ, false, MODE>::value;
-    static constexpr int occ_b = FACES ? FluxOcc<T, D, TX, TY, TZ>::value : Occ<T, D, TX, TY, TZ, true, MODE>::value;
+    static constexpr int occ_a = UOcc<T, D, TX, TY, TZ, false>::value;
+    static constexpr int occ_b = BOcc<T, D, TX, TY, TZ, false, false>::value;
     static constexpr int occ = occ_a < occ_b ? occ_a : occ_b;
 };
 
@@ -76,10 +77,11 @@ __global__ void __launch_bounds__(Tile<D, TX, TY, TZ>::NT, (PersistSmem<T, D, TX
     k_batch_persist(const PHead* __restrict__ head, const PItem* __restrict__ items, const Inst<T>* __restrict__ insts,
                     int* cur, PState* st, int nsteps, int wait_log2, int test_hook) {
     extern __shared__ __align__(128) unsigned char smem[];
+    __shared__ __align__(16) unsigned char rec_mem[sizeof(URec<T>)];
+    URec<T>& rec = *reinterpret_cast<URec<T>*>(rec_mem);
     __shared__ unsigned s_item;
     __shared__ int s_ok;
     constexpr int NT = Tile<D, TX, TY, TZ>::NT;
-    constexpr bool FACES = mode_faces(MODE);
     const int t = threadIdx.x;
     const int nitems = head->nitems;
     const unsigned total = (unsigned)nitems * (unsigned)nsteps;
@@ -134,12 +136,13 @@ __global__ void __launch_bounds__(Tile<D, TX, TY, TZ>::NT, (PersistSmem<T, D, TX
         const int c = (cur[m] + s) & 1;
         const Inst<T>& in = insts[m];
         if (it.kind == PK_A) {
-            sweep_body<T, D, TX, TY, TZ, false, MODE, true>(in.g, in.b[c], it.a, it.b, smem);
+            rec.load(in, c);
+            usweep_body<T, D, TX, TY, TZ, false, false>(rec.g, rec.b, it.a, it.b, smem);
         } else if (it.kind == PK_F) {
             for (long long k = t; k < it.count; k += NT) facec_body<T, D>(in.g, in.b[c], it.a, it.start + k);
         } else if (it.kind == PK_B) {
-            if constexpr (FACES) flux_body<T, D, TX, TY, TZ, false, false, false, true>(in.g, in.b[c], it.a, it.b, smem);
-            else sweep_body<T, D, TX, TY, TZ, true, MODE, true>(in.g, in.b[c], it.a, it.b, smem);
+            rec.load(in, c);
+            bflux_body<T, D, TX, TY, TZ, false, false, false, true>(rec.g, rec.b, it.a, it.b, smem);
         } else {
             for (long long k = t; k < it.count; k += NT) wupdate_body<T, D>(in.g, in.b[c], it.start + k);
         }

@@ -6,12 +6,13 @@ namespace cdg {
 
 int tile_count_f32(int D) { return shapes_of<float>(D).count; }
 TileShape tile_shape_f32(int D, int id) { return shapes_of<float>(D).shape(id); }
+TileShape b_tile_shape_f32(int D, int id) { return shapes_of<float>(D).b_shape(id); }
 size_t sweep_smem_f32(int D, int id) { return shapes_of<float>(D).smem(id); }
 int tile_mode_f32(int D, int id) { return shapes_of<float>(D).mode(id); }
 
-cudaError_t launch_step_f32(const Geo& g, const Inst<float>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
+cudaError_t launch_step_f32(const Geo& g, const Bufs<float>& hb, const Inst<float>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
                             const void* phi_in) {
-    return shapes_of<float>(g.D).step(g.tile_id, g, in, cur, s, ev, phi_in);
+    return shapes_of<float>(g.D).step(g.tile_id, g, hb, in, cur, s, ev, phi_in);
 }
 bool batch_persistent_f32(int D, int id) { return shapes_of<float>(D).persistent(id); }
 cudaError_t launch_batch_persist_f32(int D, int id, const PHead* h, const PItem* it, const Inst<float>* in, int* cur,

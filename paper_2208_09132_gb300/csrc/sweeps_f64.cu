@@ -7,12 +7,13 @@ namespace cdg {
 
 int tile_count_f64(int D) { return shapes_of<double>(D).count; }
 TileShape tile_shape_f64(int D, int id) { return shapes_of<double>(D).shape(id); }
+TileShape b_tile_shape_f64(int D, int id) { return shapes_of<double>(D).b_shape(id); }
 size_t sweep_smem_f64(int D, int id) { return shapes_of<double>(D).smem(id); }
 int tile_mode_f64(int D, int id) { return shapes_of<double>(D).mode(id); }
 
-cudaError_t launch_step_f64(const Geo& g, const Inst<double>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
+cudaError_t launch_step_f64(const Geo& g, const Bufs<double>& hb, const Inst<double>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
                             const void* phi_in) {
-    return shapes_of<double>(g.D).step(g.tile_id, g, in, cur, s, ev, phi_in);
+    return shapes_of<double>(g.D).step(g.tile_id, g, hb, in, cur, s, ev, phi_in);
 }
 bool batch_persistent_f64(int D, int id) { return shapes_of<double>(D).persistent(id); }
 cudaError_t launch_batch_persist_f64(int D, int id, const PHead* h, const PItem* it, const Inst<double>* in, int* cur,

@@ -7,6 +7,7 @@
 #include "launch.cuh"
 #include "lean.cuh"
 #include "persist.cuh"
+#include "bflux.cuh"
 
 namespace cdg {
 
@@ -96,6 +97,59 @@ TmaPair make_tma(const Geo& g, const void* phi_in) {
 // only) add k_faceq before the face constants and k_cellq before the W update.
 // Acceleration shapes (MODE_ACC, prepared face-store only) form the force
 // terms in k_prep and take them in k_flux.
+// Sweep B on tiles of BX x BY x BZ cells, for one instance or (BATCH) a list of items.
+template <typename T, int D, int BX, int BY, int BZ, bool SK, bool XF, bool BATCH>
+struct BLaunch {
+    using BS = BSmem<T, D, BX, BY, BZ, SK, XF>;
+    using TL = typename BS::TL;
+    static cudaError_t configure() {
+        const auto size = [](auto* kern) {
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS::bytes);
+        };
+        cudaError_t e = size(k_bflux<T, D, BX, BY, BZ, SK, true, XF>);
+        if constexpr (!SK) {
+            if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, false, XF>);
+        }
+        if constexpr (BATCH) {
+            if (!e) e = size(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF>);
+        }
+        return e;
+    }
+    static cudaError_t launch_batch(const Item* items, int n, const Inst<T>* insts, const int* cur, cudaStream_t s) {
+        return launch_pdl(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF>, dim3(n), dim3(TL::NT), BS::bytes, s, items, insts, cur);
+    }
+    static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
+    static cudaError_t launch(const Geo& g, const Bufs<T>& hb, cudaStream_t s) {
+        unsigned tiles = 1;
+        for (int a = 0; a < D; ++a) tiles *= (unsigned)((g.n[a] + TL::tdim(a) - 1) / TL::tdim(a));
+        const dim3 grid(tiles, g.G);
+        if constexpr (!SK) {
+            if (!g.nosrc)
+                return launch_pdl(k_bflux<T, D, BX, BY, BZ, false, false, XF>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
+        }
+        return launch_pdl(k_bflux<T, D, BX, BY, BZ, SK, true, XF>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
+    }
+};
+// The tile of sweep B (outside the persistent step, whose blocks are those of
+// the shape).  In FP32 CTAs of 128 threads: three per SM with up to 168
+// registers each (the chunk in flight, the next one's loads and the sums fit
+// without spills) overlap each other's barriers better than two of 256: 3D
+// 8 x 8 x 4 -> 8 x 4 x 4 12.0 -> 9.1 ps per point and step (32^3 x 24^3), 2D
+// 32 x 8 -> 32 x 4 5.94 -> 5.79 (256^2 x 32^2) and 7.98 -> 7.27 (100^2 x 101^2);
+// 16 x 8: 6.09 and 7.48.
+template <typename T, int D, int TX, int TY, int TZ>
+struct BTile {
+    static constexpr int X = TX, Y = TY, Z = TZ;
+};
+template <int TX, int TY, int TZ>
+struct BTile<float, 2, TX, TY, TZ> {
+    static constexpr int X = 32, Y = 4, Z = 1;
+};
+template <int TX, int TY, int TZ>
+struct BTile<float, 3, TX, TY, TZ> {
+    static constexpr int X = 8, Y = 4, Z = 4;
+};
+
 // The number of CTAs of a persistent launch: every SM at the occupancy the
 // kernel reaches (more would only wait for a slot).
 template <typename K>
@@ -129,11 +183,19 @@ struct Shape {
     // batched steps: the fused shapes (incl. Shakhov) and the acceleration
     // shapes (their pre-pass is batched too)
     static constexpr bool BATCH = SRC == MODE_FUSED || ACC;
+    using BT = BTile<T, D, TX, TY, TZ>;
+    using BL = BLaunch<T, D, BT::X, BT::Y, BT::Z, SK, false, BATCH>;
+    // sweep A with upwind owners (usweep.cuh)
+    static constexpr bool UP = mode_upwind(MODE);
+    using US = USmem<T, D, TX, TY, TZ, false, SK>;
+    // sweep B of the face-store shapes: bflux.cuh's, or k_flux with the acceleration
+    static constexpr bool BF = FACES && !ACC;
 
     // dynamic shared memory of the larger of the two sweeps
     static size_t smem_bytes() {
-        const size_t b = FACES ? FS::bytes : SM::bytes(true);
-        return SM::bytes(false) > b ? SM::bytes(false) : b;
+        const size_t a = UP ? US::bytes : SM::bytes(false);
+        const size_t b = BF ? BL::BS::bytes : (FACES ? FS::bytes : SM::bytes(true));
+        return a > b ? a : b;
     }
 
     static cudaError_t configure() {
@@ -143,7 +205,9 @@ struct Shape {
         if ((e = cudaFuncSetAttribute(k_sweep<T, D, TX, TY, TZ, false, MODE>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
             return e;
-        if constexpr (FACES) {
+        if constexpr (BF) {
+            if ((e = BL::configure())) return e;
+        } else if constexpr (FACES) {
             if ((e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, SK, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                           (int)FS::bytes)))
                 return e;
@@ -152,10 +216,22 @@ struct Shape {
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(true))))
                 return e;
         }
-        if constexpr (NS) {
+        if constexpr (UP) {
+            const auto size = [](auto* kern) {
+                return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)US::bytes);
+            };
+            if ((e = size(k_usweep<T, D, TX, TY, TZ, false, true, SK>)) ||
+                (e = size(k_usweep_batch<T, D, TX, TY, TZ, false, SK, SK>)))
+                return e;
+            if constexpr (NS) {
+                if ((e = size(k_usweep<T, D, TX, TY, TZ, false, false>))) return e;
+            }
+        } else if constexpr (NS) {
             if ((e = cudaFuncSetAttribute(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
                 return e;
+        }
+        if constexpr (NS && ACC) {
             if ((e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, false, ACC, true>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)))
                 return e;
@@ -166,14 +242,16 @@ struct Shape {
                 return e;
         }
         if constexpr (BATCH) {
-            if ((e = cudaFuncSetAttribute(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
-                return e;
-            if constexpr (FACES) {
+            if constexpr (!UP || SK) {
+                if ((e = cudaFuncSetAttribute(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>,
+                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
+                    return e;
+            }
+            if constexpr (FACES && !BF) {
                 if ((e = cudaFuncSetAttribute(k_flux_batch<T, D, TX, TY, TZ, SK, ACC>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)))
                     return e;
-            } else {
+            } else if constexpr (!FACES) {
                 if ((e = cudaFuncSetAttribute(k_sweep_batch<T, D, TX, TY, TZ, true, MODE>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(true))))
                     return e;
@@ -183,7 +261,7 @@ struct Shape {
         return cudaSuccess;
     }
 
-    static cudaError_t step(const Geo& g, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
+    static cudaError_t step(const Geo& g, const Bufs<T>& hb, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
                             const void* phi_in) {
         cudaError_t e = configure();
         if (e) return e;
@@ -198,14 +276,24 @@ struct Shape {
                                 shslope_smem_bytes<T, D, TX, TY, TZ, SK>(), s, in, cur)))
                 return e;
         }
-        const TmaPair tma = make_tma<T, D, typename SM::TL>(g, SM::stage(false) ? phi_in : nullptr);
-        const bool ns = NS && g.nosrc;
-        if constexpr (NS) {
-            if (ns)
-                e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>, grid, dim3(TL::NT), SM::bytes(false), s, in,
-                               cur, tma);
+        const bool ns = NS && g.nosrc, up = UP && g.upw && !g.wait_test;
+        if constexpr (UP) {
+            if (up && (ns || SK)) {
+                e = launch_pdl(k_usweep<T, D, TX, TY, TZ, false, true, SK>, grid, dim3(TL::NT), US::bytes_of(g), s, g, hb);
+            } else if (up) {
+                if constexpr (NS) e = launch_pdl(k_usweep<T, D, TX, TY, TZ, false, false>, grid, dim3(TL::NT), US::bytes_of(g), s, g, hb);
+            }
         }
-        if (!ns) e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE>, grid, dim3(TL::NT), SM::bytes(false), s, in, cur, tma);
+        if (!up) {      // (a shape with upwind owners: the Shakhov model with a node at 0, and the wait hook)
+            const TmaPair tma = make_tma<T, D, typename SM::TL>(g, SM::stage(false) ? phi_in : nullptr);
+            if constexpr (NS && !UP) {
+                if (ns)
+                    e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>, grid, dim3(TL::NT), SM::bytes(false), s, in,
+                                   cur, tma);
+            }
+            if (!ns || UP)
+                e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE>, grid, dim3(TL::NT), SM::bytes(false), s, in, cur, tma);
+        }
         if (e) return e;
         if (ev) cudaEventRecord(ev[1], s);
         if constexpr (SK) {
@@ -221,7 +309,9 @@ struct Shape {
             if ((e = launch_pdl(k_facec<T, D>, fgrid, dim3(kSmallBlock), 0, s, in, cur))) return e;
         }
         if (ev) cudaEventRecord(ev[2], s);
-        if constexpr (NS) {
+        if constexpr (BF) {
+            e = BL::launch(g, hb, s);
+        } else if constexpr (NS) {
             if (ns) e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, ACC, true>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
             else e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, ACC>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
         } else if constexpr (FACES)
@@ -241,7 +331,7 @@ struct Shape {
         return cudaGetLastError();
     }
 
-    static cudaError_t sweep_batch(bool B, const Item* items, int n, const Inst<T>* insts, const int* cur,
+    static cudaError_t sweep_batch(bool B, bool up, const Item* items, int n, const Inst<T>* insts, const int* cur,
                                    cudaStream_t s) {
         if constexpr (!BATCH) {
             return cudaErrorNotSupported;
@@ -249,10 +339,20 @@ struct Shape {
             cudaError_t e = configure();
             if (e) return e;
             if (n <= 0) return cudaSuccess;
-            if (!B)
-                return launch_pdl(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>, dim3(n), dim3(TL::NT), SM::bytes(false),
-                                  s, items, insts, cur);
-            if constexpr (FACES)
+            if (!B) {
+                if constexpr (UP) {
+                    if (up)
+                        return launch_pdl(k_usweep_batch<T, D, TX, TY, TZ, false, SK, SK>, dim3(n), dim3(TL::NT), US::bytes,
+                                          s, items, insts, cur);
+                }
+                if constexpr (!UP || SK)
+                    return launch_pdl(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>, dim3(n), dim3(TL::NT),
+                                      SM::bytes(false), s, items, insts, cur);
+                return cudaErrorNotSupported;
+            }
+            if constexpr (BF)
+                return BL::launch_batch(items, n, insts, cur, s);
+            else if constexpr (FACES)
                 return launch_pdl(k_flux_batch<T, D, TX, TY, TZ, SK, ACC>, dim3(n), dim3(TL::NT), FS::bytes, s, items,
                                   insts, cur);
             else
@@ -262,6 +362,10 @@ struct Shape {
     }
 
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
+    static TileShape b_shape() {
+        if constexpr (BF) return BL::shape();
+        else return shape();
+    }
 
     static constexpr bool persistent = PB;
     static cudaError_t persist(const PHead* head, const PItem* items, const Inst<T>* insts, int* cur, PState* st,
@@ -287,60 +391,48 @@ struct Shape {
     }
 };
 
-// A lean shape (lean.cuh): sweep A k_lsweep, face constants (with the face
+// A lean shape (lean.cuh): sweep A k_usweep, face constants (with the face
 // factor tables when XF), sweep B k_lflux (XF) or k_flux, W update (with the
 // cell factor tables).  Single instances take the sweeps without the b-source
 // terms when the instance has none (Pr = 1); batched launches keep the general
 // ones.
 template <typename T, int D, int TX, int TY, int TZ, bool XF = true>
 struct LeanShape {
-    using LA = LeanA<T, D, TX, TY, TZ>;
-    using LB = LeanB<T, D, TX, TY, TZ>;
-    using FS = FluxSmem<T, D, TX, TY, TZ>;
+    using LA = USmem<T, D, TX, TY, TZ, true>;
+    using BT = BTile<T, D, TX, TY, TZ>;
+    using BL = BLaunch<T, D, BT::X, BT::Y, BT::Z, false, XF, true>;
     using TL = Tile<D, TX, TY, TZ>;
     static constexpr int mode = MODE_LEAN | MODE_FACES | (XF ? MODE_XF : 0);
-    static constexpr size_t b_bytes = XF ? LB::bytes : FS::bytes;
-    static size_t smem_bytes() { return LA::bytes > b_bytes ? LA::bytes : b_bytes; }
+    static size_t smem_bytes() { return LA::bytes > BL::BS::bytes ? LA::bytes : BL::BS::bytes; }
 
     static cudaError_t configure() {
         static bool done = false;
         if (done) return cudaSuccess;
         cudaError_t e;
-        if ((e = cudaFuncSetAttribute(k_lsweep<T, D, TX, TY, TZ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)LA::bytes)) ||
-            (e = cudaFuncSetAttribute(k_lsweep<T, D, TX, TY, TZ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)LA::bytes)) ||
-            (e = cudaFuncSetAttribute(k_lsweep_batch<T, D, TX, TY, TZ, false>,
-                                      cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LA::bytes)))
+        const auto size = [](auto* kern, size_t bytes) {
+            return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        };
+        if ((e = size(k_usweep<T, D, TX, TY, TZ, true, false>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, true>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, false, false, D != 3>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, true, false, D != 3>, LA::bytes)) ||
+            (e = size(k_usweep_batch<T, D, TX, TY, TZ, true, false>, LA::bytes)) ||
+            (e = BL::configure()))
             return e;
-        if constexpr (XF) {
-            if ((e = cudaFuncSetAttribute(k_lflux<T, D, TX, TY, TZ, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)LB::bytes)) ||
-                (e = cudaFuncSetAttribute(k_lflux<T, D, TX, TY, TZ, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)LB::bytes)) ||
-                (e = cudaFuncSetAttribute(k_lflux_batch<T, D, TX, TY, TZ, false>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LB::bytes)))
-                return e;
-        } else {
-            if ((e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, false, false, false>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)) ||
-                (e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, false, false, true>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)) ||
-                (e = cudaFuncSetAttribute(k_flux_batch<T, D, TX, TY, TZ>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)FS::bytes)))
-                return e;
-        }
         done = true;
         return cudaSuccess;
     }
 
-    static cudaError_t step(const Geo& g, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev, const void*) {
+    static cudaError_t step(const Geo& g, const Bufs<T>& hb, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
+                            const void*) {
         cudaError_t e = configure();
         if (e) return e;
         const dim3 grid(g.tiles[0] * g.tiles[1] * g.tiles[2], g.G);
         if (ev) cudaEventRecord(ev[0], s);
-        if (g.nosrc) e = launch_pdl(k_lsweep<T, D, TX, TY, TZ, true>, grid, dim3(TL::NT), LA::bytes, s, in, cur);
-        else e = launch_pdl(k_lsweep<T, D, TX, TY, TZ, false>, grid, dim3(TL::NT), LA::bytes, s, in, cur);
+        const auto a = [&](auto* kern) { return launch_pdl(kern, grid, dim3(TL::NT), LA::bytes_of(g), s, g, hb); };
+        if (g.mixed) e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true>) : a(k_usweep<T, D, TX, TY, TZ, true, false>);
+        else e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true, false, D != 3>)
+                         : a(k_usweep<T, D, TX, TY, TZ, true, false, false, D != 3>);
         if (e) return e;
         if (ev) cudaEventRecord(ev[1], s);
         {
@@ -350,14 +442,7 @@ struct LeanShape {
             if ((e = launch_pdl(k_facec<T, D>, fgrid, dim3(kSmallBlock), 0, s, in, cur))) return e;
         }
         if (ev) cudaEventRecord(ev[2], s);
-        if constexpr (XF) {
-            if (g.nosrc) e = launch_pdl(k_lflux<T, D, TX, TY, TZ, true>, grid, dim3(TL::NT), LB::bytes, s, in, cur);
-            else e = launch_pdl(k_lflux<T, D, TX, TY, TZ, false>, grid, dim3(TL::NT), LB::bytes, s, in, cur);
-        } else {
-            if (g.nosrc) e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, false, true>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
-            else e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, false, false>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
-        }
-        if (e) return e;
+        if ((e = BL::launch(g, hb, s))) return e;
         if (ev) cudaEventRecord(ev[3], s);
         if ((e = launch_pdl(k_wupdate<T, D>, dim3((unsigned)((g.Nc + kSmallBlock - 1) / kSmallBlock)), dim3(kSmallBlock),
                             0, s, in, cur)))
@@ -366,22 +451,19 @@ struct LeanShape {
         return cudaGetLastError();
     }
 
-    static cudaError_t sweep_batch(bool B, const Item* items, int n, const Inst<T>* insts, const int* cur,
+    static cudaError_t sweep_batch(bool B, bool, const Item* items, int n, const Inst<T>* insts, const int* cur,
                                    cudaStream_t s) {
         cudaError_t e = configure();
         if (e) return e;
         if (n <= 0) return cudaSuccess;
         if (!B)
-            return launch_pdl(k_lsweep_batch<T, D, TX, TY, TZ, false>, dim3(n), dim3(TL::NT), LA::bytes, s, items, insts,
-                              cur);
-        if constexpr (XF)
-            return launch_pdl(k_lflux_batch<T, D, TX, TY, TZ, false>, dim3(n), dim3(TL::NT), LB::bytes, s, items, insts,
-                              cur);
-        else
-            return launch_pdl(k_flux_batch<T, D, TX, TY, TZ>, dim3(n), dim3(TL::NT), FS::bytes, s, items, insts, cur);
+            return launch_pdl(k_usweep_batch<T, D, TX, TY, TZ, true, false>, dim3(n), dim3(TL::NT), LA::bytes, s, items,
+                              insts, cur);
+        return BL::launch_batch(items, n, insts, cur, s);
     }
 
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
+    static TileShape b_shape() { return BL::shape(); }
 
     static constexpr bool persistent = false;
     static cudaError_t persist(const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t) {
@@ -396,14 +478,15 @@ template <>
 struct ShapeList<> {
     static constexpr int count = 0;
     template <typename T>
-    static cudaError_t step(int, const Geo&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*) {
+    static cudaError_t step(int, const Geo&, const Bufs<T>&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*) {
         return cudaErrorInvalidValue;
     }
     template <typename T>
-    static cudaError_t sweep_batch(int, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t) {
+    static cudaError_t sweep_batch(int, bool, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t) {
         return cudaErrorInvalidValue;
     }
     static TileShape shape(int) { return {{0, 0, 0}}; }
+    static TileShape b_shape(int) { return {{0, 0, 0}}; }
     static size_t smem(int) { return 0; }
     static int mode(int) { return 0; }
     static bool persistent(int) { return false; }
@@ -418,17 +501,19 @@ struct ShapeList<H, R...> {
     using Rest = ShapeList<R...>;
     static constexpr int count = 1 + Rest::count;
     template <typename T>
-    static cudaError_t step(int id, const Geo& g, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
+    static cudaError_t step(int id, const Geo& g, const Bufs<T>& hb, const Inst<T>* in, int cur, cudaStream_t s, cudaEvent_t* ev,
                             const void* phi_in) {
-        return id == 0 ? H::step(g, in, cur, s, ev, phi_in)
-                       : Rest::template step<T>(id - 1, g, in, cur, s, ev, phi_in);
+        return id == 0 ? H::step(g, hb, in, cur, s, ev, phi_in)
+                       : Rest::template step<T>(id - 1, g, hb, in, cur, s, ev, phi_in);
     }
     template <typename T>
-    static cudaError_t sweep_batch(int id, bool B, const Item* it, int n, const Inst<T>* in, const int* cur,
+    static cudaError_t sweep_batch(int id, bool B, bool up, const Item* it, int n, const Inst<T>* in, const int* cur,
                                    cudaStream_t s) {
-        return id == 0 ? H::sweep_batch(B, it, n, in, cur, s) : Rest::template sweep_batch<T>(id - 1, B, it, n, in, cur, s);
+        return id == 0 ? H::sweep_batch(B, up, it, n, in, cur, s)
+                       : Rest::template sweep_batch<T>(id - 1, B, up, it, n, in, cur, s);
     }
     static TileShape shape(int id) { return id == 0 ? H::shape() : Rest::shape(id - 1); }
+    static TileShape b_shape(int id) { return id == 0 ? H::b_shape() : Rest::b_shape(id - 1); }
     static size_t smem(int id) { return id == 0 ? H::smem_bytes() : Rest::smem(id - 1); }
     static int mode(int id) { return id == 0 ? H::mode : Rest::mode(id - 1); }
     static bool persistent(int id) { return id == 0 ? H::persistent : Rest::persistent(id - 1); }
@@ -447,16 +532,17 @@ template <typename T>
 struct ShapeOps {
     int count;
     TileShape (*shape)(int);
+    TileShape (*b_shape)(int);      // the tile of sweep B's batched items
     size_t (*smem)(int);
     int (*mode)(int);
     bool (*persistent)(int);
-    cudaError_t (*step)(int, const Geo&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*);
-    cudaError_t (*sweep_batch)(int, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t);
+    cudaError_t (*step)(int, const Geo&, const Bufs<T>&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*);
+    cudaError_t (*sweep_batch)(int, bool, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t);
     cudaError_t (*persist)(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t);
 };
 template <typename T, typename L>
 ShapeOps<T> ops_of() {
-    return {L::count, &L::shape, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
+    return {L::count, &L::shape, &L::b_shape, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
             &L::template sweep_batch<T>, &L::template persist<T>};
 }
 const ShapeOps<float>& shapes_f32_1();
@@ -500,7 +586,7 @@ cudaError_t run_batch_step(const BatchPlan& p, const Inst<T>* insts, int* cur, c
         if (e) return e;
     }
     for (int k = 0; k < p.ntile; ++k)
-        if ((e = ops.sweep_batch(p.tile_id[k], false, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
+        if ((e = ops.sweep_batch(p.tile_id[k], false, p.upw[k], p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
             return e;
     if ((e = launch_rawq_batch<T>(p.D, p.faceq_items, p.n_faceq, insts, cur, s))) return e;
     if (p.n_face > 0) {
@@ -512,7 +598,7 @@ cudaError_t run_batch_step(const BatchPlan& p, const Inst<T>* insts, int* cur, c
         if (e) return e;
     }
     for (int k = 0; k < p.ntile; ++k)
-        if ((e = ops.sweep_batch(p.tile_id[k], true, p.sweep_items[k], p.n_sweep[k], insts, cur, s)))
+        if ((e = ops.sweep_batch(p.tile_id[k], true, p.upw[k], p.sweep_b_items[k], p.n_sweep_b[k], insts, cur, s)))
             return e;
     if ((e = launch_rawq_batch<T>(p.D, p.cellq_items, p.n_cellq, insts, cur, s))) return e;
     if (p.n_cell > 0) {
