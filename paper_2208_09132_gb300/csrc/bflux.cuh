@@ -197,7 +197,7 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
 #pragma unroll
         for (int m = 0; m < NM; ++m) RS[m * NX + t].zero();
 
-    T hL = SK ? (T)(0.5 * (3.0 - D + g.K)) : T(0), dxi = GQ ? (T)g.dxi[0] : T(0);
+    T hL = SK ? g.consts<T>().ceb : T(0), dxi = GQ ? (T)g.dxi[0] : T(0);
     if (SK) keep(hL);
     if (GQ) keep(dxi);
     if (t == 0) {

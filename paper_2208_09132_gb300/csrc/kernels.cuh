@@ -59,6 +59,14 @@ struct TmaPair {
     int on;
 };
 
+// Constants of an instance in a storage precision, formed once on the host: the
+// conversions from double (and the division in cT) would run on the FP64 pipe
+// for every cell and face.
+template <typename R>
+struct GeoConst {
+    R mu_ref, T_ref, omega, Pr, dt, hdt, hh, ceb;      // hdt = dt/2, hh = h/2, ceb = (3 - D + K)/2
+};
+
 // Problem geometry and physics, passed by value to every kernel.
 struct Geo {
     int D;
@@ -77,7 +85,15 @@ struct Geo {
     double hdx[3];    // h / dx_a
     double idx[3];    // 1 / dx_a
     double dt, h;
-    double K, R, mu_ref, T_ref, omega, Pr;
+    double K, R, Pr;
+    double cT;        // 2 / ((K + 3) R): T = cT (E - u^2/2)
+    GeoConst<float> cf;
+    GeoConst<double> cd;
+    template <typename T>
+    __host__ __device__ __forceinline__ const GeoConst<T>& consts() const {
+        if constexpr (sizeof(T) == 4) return cf;
+        else return cd;
+    }
     int shakhov;      // collision model: 0 the two relaxation times of Sec. 2, 1 the Shakhov S-model
     int accel;        // a uniform external acceleration is on (eqs. gsource, bsource)
     double acc[3];    // its components a_b (0 beyond D)
@@ -292,7 +308,7 @@ __device__ __forceinline__ Macro macro_of(const Geo& g, const double* W) {
     }
     const double E = dmul(W[1 + g.D], irho);
     // T = (gamma - 1)/R (E - u^2/2), gamma = (K+5)/(K+3)
-    m.T = dmul(ddiv(2.0, dmul(dadd(g.K, 3.0), g.R)), dsub(E, dmul(0.5, u2)));
+    m.T = dmul(g.cT, dsub(E, dmul(0.5, u2)));
     m.RT = dmul(g.R, m.T);
     return m;
 }
@@ -310,14 +326,15 @@ template <typename R>
 __device__ __forceinline__ Relax<R> relax_of(const Geo& g, const Macro& m) {
     using A = Ar<R>;
     Relax<R> r;
-    const R mu = A::mul((R)g.mu_ref, visc_power<R>(A::div((R)m.T, (R)g.T_ref), (R)g.omega));
+    const GeoConst<R>& c = g.consts<R>();
+    const R mu = A::mul(c.mu_ref, visc_power<R>(A::div((R)m.T, c.T_ref), c.omega));
     r.itg = A::div(A::mul((R)m.rho, (R)m.RT), mu);
     if (g.shakhov) {           // one relaxation time, no b-source
         r.itb = r.itg;
         r.itbg = R(0);
     } else {
-        r.itb = A::mul((R)g.Pr, r.itg);
-        r.itbg = A::mul(A::sub((R)g.Pr, R(1)), r.itg);
+        r.itb = A::mul(c.Pr, r.itg);
+        r.itbg = A::mul(A::sub(c.Pr, R(1)), r.itg);
     }
     return r;
 }
@@ -376,7 +393,7 @@ __device__ __forceinline__ void eq_consts(const Geo& g, const Macro& m, T u[3], 
     const T RT = (T)m.RT;
     cexp = A::div((T)(-0.5 * Num<T>::cexp_scale()), RT);
     pref = A::mul((T)m.rho, gauss_norm<T>(A::mul((T)(2.0 * 3.14159265358979323846), RT), g.D));
-    eb = A::mul((T)(0.5 * (3.0 - g.D + g.K)), RT);
+    eb = A::mul(g.consts<T>().ceb, RT);
     hu2 = (T)dmul(0.5, u2);
 }
 
@@ -390,7 +407,7 @@ __device__ __forceinline__ void make_cell(const Geo& g, const double* W, const d
     const Relax<T> r = relax_of<T>(g, m);
     eq_consts<T>(g, m, c.u, c.cexp, c.pref, c.eb, c.hu2);
     shakhov_consts<T>(g, m, q, c.sq, c.e2);
-    const T dt = (T)g.dt, hh = (T)(0.5 * g.h), hdt = (T)(0.5 * g.dt);
+    const T dt = g.consts<T>().dt, hh = g.consts<T>().hh, hdt = g.consts<T>().hdt;
     const T xg = A::mul(hdt, r.itg), xb = A::mul(hdt, r.itb);
     const T fa_g = A::div(T(1), A::add(T(1), xg)), fa_b = A::div(T(1), A::add(T(1), xb));
     c.fa_g = fa_g;
@@ -414,7 +431,7 @@ __device__ __forceinline__ void make_face(const Geo& g, const double* W, const d
     const Relax<T> r = relax_of<T>(g, m);
     eq_consts<T>(g, m, f.u, f.cexp, f.pref, f.eb, f.hu2);
     shakhov_consts<T>(g, m, q, f.sq, f.e2);
-    const T hh = (T)(0.5 * g.h);
+    const T hh = g.consts<T>().hh;
     f.al_g = A::div(T(1), A::add(T(1), A::mul(hh, r.itg)));
     f.al_b = A::div(T(1), A::add(T(1), A::mul(hh, r.itb)));
     f.gam_b = A::mul(A::mul(hh, r.itbg), f.al_b);

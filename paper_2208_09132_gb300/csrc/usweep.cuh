@@ -125,7 +125,7 @@ __device__ __noinline__ void phibar_at(const Geo& g, const Bufs<T>& bf, int q0, 
         }
         lean_geq4<T, D>(g, dir ? bf.xc0 : bf.xc, g.Nc, c, refl, vt, R, ge);
     }
-    const T hL = (T)(0.5 * (3.0 - D + g.K));
+    const T hL = g.consts<T>().ceb;
 #pragma unroll
     for (int v = 0; v < VC; ++v) {
         T z = -cs.hu2, be;
@@ -492,7 +492,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         ends |= (valid && qa[a] == 0 ? 1 : 0) << (2 * a);
         ends |= (valid && qa[a] == g.n[a] - 1 ? 2 : 0) << (2 * a);
     }
-    const T hL = SK ? (T)(0.5 * (3.0 - D + g.K)) : T(0), dxi = gauss_ratio<T, D>() ? (T)g.dxi[0] : T(0);
+    const T hL = SK ? g.consts<T>().ceb : T(0), dxi = gauss_ratio<T, D>() ? (T)g.dxi[0] : T(0);
     auto fstr = [&](int a) { return a == 0 ? 1 : (a == 1 ? g.fn[1][0] : g.fn[2][0] * g.fn[2][1]); };
 
     Sums<T, D * NM> acc;
