@@ -150,12 +150,25 @@ void set_tiles(cdugks* h, int id) {
 int groups_for(const cdugks* h, int requested) {
     const Geo& g = h->g;
     if (requested > 0) return std::min(requested, g.NVT);
-    // enough CTAs for a few full waves over 152 SMs (at least 2 resident per SM)
+    // The split of least cost, in chunks of one CTA's work: the chunks, times how
+    // far the last wave of CTAs (152 SMs, as many per SM as sweep A runs) is from
+    // full, plus what every group adds (its partial sums in the face and cell
+    // kernels, the CTAs' prologues: about 3.5 chunks in FP32, 0.5 of the slower FP64
+    // ones).
     const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2];
-    const long long want = 152LL * 2 * 4;
-    long long G = (want + tiles - 1) / tiles;
-    G = std::max(1LL, std::min<long long>(G, g.NVT));
-    G = std::min<long long>(G, 64);
+    const long long slots = 152LL * (h->prec == CDUGKS_FP32 ? cdg::sweep_a_ctas_f32(g.D, g.tile_id)
+                                                            : cdg::sweep_a_ctas_f64(g.D, g.tile_id));
+    const double per_group = h->prec == CDUGKS_FP32 ? 3.5 : 0.5;
+    long long G = 1;
+    double best = 0.0;
+    for (long long n = 1; n <= std::min(g.NVT, 64); ++n) {
+        const long long ctas = tiles * n, waves = (ctas + slots - 1) / slots;
+        const double cost = (double)g.NVT * (double)(waves * slots) / (double)ctas + per_group * (double)n;
+        if (n == 1 || cost < best) {
+            best = cost;
+            G = n;
+        }
+    }
     return (int)G;
 }
 

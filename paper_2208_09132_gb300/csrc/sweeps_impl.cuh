@@ -366,6 +366,10 @@ struct Shape {
         if constexpr (BF) return BL::shape();
         else return shape();
     }
+    static int a_ctas() {
+        if constexpr (UP) return UOcc<T, D, TX, TY, TZ, false, SK>::value;
+        else return Occ<T, D, TX, TY, TZ, false, MODE>::value;
+    }
 
     static constexpr bool persistent = PB;
     static cudaError_t persist(const PHead* head, const PItem* items, const Inst<T>* insts, int* cur, PState* st,
@@ -468,6 +472,7 @@ struct LeanShape {
     static constexpr bool persistent = false;
     static cudaError_t persist(const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t) {
         return cudaErrorNotSupported;
+    static int a_ctas() { return UOcc<T, D, TX, TY, TZ, true>::value; }
     }
 };
 
@@ -491,6 +496,7 @@ struct ShapeList<> {
     static int mode(int) { return 0; }
     static bool persistent(int) { return false; }
     template <typename T>
+    static int a_ctas(int) { return 1; }
     static cudaError_t persist(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int,
                                cudaStream_t) {
         return cudaErrorInvalidValue;
@@ -518,6 +524,7 @@ struct ShapeList<H, R...> {
     static int mode(int id) { return id == 0 ? H::mode : Rest::mode(id - 1); }
     static bool persistent(int id) { return id == 0 ? H::persistent : Rest::persistent(id - 1); }
     template <typename T>
+    static int a_ctas(int id) { return id == 0 ? H::a_ctas() : Rest::a_ctas(id - 1); }
     static cudaError_t persist(int id, const PHead* h, const PItem* it, const Inst<T>* in, int* cur, PState* st, int n,
                                int w, int th, cudaStream_t s) {
         return id == 0 ? H::persist(h, it, in, cur, st, n, w, th, s)
@@ -537,12 +544,13 @@ struct ShapeOps {
     int (*mode)(int);
     bool (*persistent)(int);
     cudaError_t (*step)(int, const Geo&, const Bufs<T>&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*);
+    int (*a_ctas)(int);             // CTAs of sweep A per SM
     cudaError_t (*sweep_batch)(int, bool, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t);
     cudaError_t (*persist)(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t);
 };
 template <typename T, typename L>
 ShapeOps<T> ops_of() {
-    return {L::count, &L::shape, &L::b_shape, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
+    return {L::count, &L::shape, &L::b_shape, &L::a_ctas, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
             &L::template sweep_batch<T>, &L::template persist<T>};
 }
 const ShapeOps<float>& shapes_f32_1();
