@@ -607,6 +607,14 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     g.K = phys->K;
     g.R = phys->R;
     g.Pr = phys->Pr;
+    g.cT = 2.0 / ((g.K + 3.0) * g.R);
+    const auto consts = [&](auto& c) {
+        using V = std::decay_t<decltype(c.Pr)>;
+        c = {(V)phys->mu_ref, (V)phys->T_ref, (V)phys->omega, (V)phys->Pr, (V)g.dt, (V)(0.5 * g.dt), (V)(0.5 * g.h),
+             (V)(0.5 * (3.0 - D + g.K))};
+    };
+    consts(g.cf);
+    consts(g.cd);
     // with Pr = 1 the TEDDF b-source coefficient (Pr - 1)/tau vanishes exactly
     g.nosrc = phys->Pr == 1.0;
     g.mirror = 1;
@@ -620,14 +628,6 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     set_groups(h, h->gcap);
     make_layout(h);
     h->stream = nullptr;
-    g.cT = 2.0 / ((g.K + 3.0) * g.R);
-    const auto consts = [&](auto& c) {
-        using V = std::decay_t<decltype(c.Pr)>;
-        c = {(V)phys->mu_ref, (V)phys->T_ref, (V)phys->omega, (V)phys->Pr, (V)g.dt, (V)(0.5 * g.dt), (V)(0.5 * g.h),
-             (V)(0.5 * (3.0 - D + g.K))};
-    };
-    consts(g.cf);
-    consts(g.cd);
     h->cur = 0;
     *out = h;
     return CDUGKS_OK;

@@ -416,10 +416,12 @@ struct LeanShape {
         const auto size = [](auto* kern, size_t bytes) {
             return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
         };
-        if ((e = size(k_usweep<T, D, TX, TY, TZ, true, false>, LA::bytes)) ||
+        if ((e = size(k_usweep<T, D, TX, TY, TZ, true, false, false, false>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, true, false, false>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, false>, LA::bytes)) ||
             (e = size(k_usweep<T, D, TX, TY, TZ, true, true>, LA::bytes)) ||
-            (e = size(k_usweep<T, D, TX, TY, TZ, true, false, false, D != 3>, LA::bytes)) ||
-            (e = size(k_usweep<T, D, TX, TY, TZ, true, true, false, D != 3>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, false, false, true, false>, LA::bytes)) ||
+            (e = size(k_usweep<T, D, TX, TY, TZ, true, true, false, true, false>, LA::bytes)) ||
             (e = size(k_usweep_batch<T, D, TX, TY, TZ, true, false>, LA::bytes)) ||
             (e = BL::configure()))
             return e;
@@ -434,9 +436,11 @@ struct LeanShape {
         const dim3 grid(g.tiles[0] * g.tiles[1] * g.tiles[2], g.G);
         if (ev) cudaEventRecord(ev[0], s);
         const auto a = [&](auto* kern) { return launch_pdl(kern, grid, dim3(TL::NT), LA::bytes_of(g), s, g, hb); };
-        if (g.mixed) e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true>) : a(k_usweep<T, D, TX, TY, TZ, true, false>);
-        else e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true, false, D != 3>)
-                         : a(k_usweep<T, D, TX, TY, TZ, true, false, false, D != 3>);
+        if (!g.xal) e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true, false, true, false>)
+                                : a(k_usweep<T, D, TX, TY, TZ, true, false, false, true, false>);
+        else if (g.mixed) e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true>) : a(k_usweep<T, D, TX, TY, TZ, true, false>);
+        else e = g.nosrc ? a(k_usweep<T, D, TX, TY, TZ, true, true, false, false>)
+                         : a(k_usweep<T, D, TX, TY, TZ, true, false, false, false>);
         if (e) return e;
         if (ev) cudaEventRecord(ev[1], s);
         {
@@ -468,11 +472,11 @@ struct LeanShape {
 
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
     static TileShape b_shape() { return BL::shape(); }
+    static int a_ctas() { return UOcc<T, D, TX, TY, TZ, true>::value; }
 
     static constexpr bool persistent = false;
     static cudaError_t persist(const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t) {
         return cudaErrorNotSupported;
-    static int a_ctas() { return UOcc<T, D, TX, TY, TZ, true>::value; }
     }
 };
 
@@ -492,11 +496,11 @@ struct ShapeList<> {
     }
     static TileShape shape(int) { return {{0, 0, 0}}; }
     static TileShape b_shape(int) { return {{0, 0, 0}}; }
+    static int a_ctas(int) { return 1; }
     static size_t smem(int) { return 0; }
     static int mode(int) { return 0; }
     static bool persistent(int) { return false; }
     template <typename T>
-    static int a_ctas(int) { return 1; }
     static cudaError_t persist(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int,
                                cudaStream_t) {
         return cudaErrorInvalidValue;
@@ -520,11 +524,11 @@ struct ShapeList<H, R...> {
     }
     static TileShape shape(int id) { return id == 0 ? H::shape() : Rest::shape(id - 1); }
     static TileShape b_shape(int id) { return id == 0 ? H::b_shape() : Rest::b_shape(id - 1); }
+    static int a_ctas(int id) { return id == 0 ? H::a_ctas() : Rest::a_ctas(id - 1); }
     static size_t smem(int id) { return id == 0 ? H::smem_bytes() : Rest::smem(id - 1); }
     static int mode(int id) { return id == 0 ? H::mode : Rest::mode(id - 1); }
     static bool persistent(int id) { return id == 0 ? H::persistent : Rest::persistent(id - 1); }
     template <typename T>
-    static int a_ctas(int id) { return id == 0 ? H::a_ctas() : Rest::a_ctas(id - 1); }
     static cudaError_t persist(int id, const PHead* h, const PItem* it, const Inst<T>* in, int* cur, PState* st, int n,
                                int w, int th, cudaStream_t s) {
         return id == 0 ? H::persist(h, it, in, cur, st, n, w, th, s)
@@ -540,11 +544,11 @@ struct ShapeOps {
     int count;
     TileShape (*shape)(int);
     TileShape (*b_shape)(int);      // the tile of sweep B's batched items
+    int (*a_ctas)(int);             // CTAs of sweep A per SM
     size_t (*smem)(int);
     int (*mode)(int);
     bool (*persistent)(int);
     cudaError_t (*step)(int, const Geo&, const Bufs<T>&, const Inst<T>*, int, cudaStream_t, cudaEvent_t*, const void*);
-    int (*a_ctas)(int);             // CTAs of sweep A per SM
     cudaError_t (*sweep_batch)(int, bool, bool, const Item*, int, const Inst<T>*, const int*, cudaStream_t);
     cudaError_t (*persist)(int, const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t);
 };

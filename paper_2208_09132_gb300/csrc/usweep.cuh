@@ -67,8 +67,12 @@ struct USmem {
     static constexpr size_t rec_bytes = 4 * kVisitInts + kVisitVecs * sizeof(V4<T>);
     static constexpr size_t mix_bytes = (size_t)mixed_axes(D) * NT * ((2 + D) * sizeof(Kahan<T>) + sizeof(V4<T>));
     static constexpr size_t bytes = (nP + nCC) * sizeof(V4<T>) + RING * rec_bytes + mix_bytes;
-    // (an instance without mixed visits leaves those sums to L1)
-    static size_t bytes_of(const Geo& g) { return g.mixed ? bytes : bytes - mix_bytes; }
+    // 3D instances without mixed visits keep the cells' numbers there instead, for
+    // the registers; the others in registers, for the size: two CTAs of up to 97
+    // KB leave L1 60 KB, larger ones 28 KB (the mixed sweep 11.9 -> 13.7 ps per point)
+    static constexpr size_t cell_bytes = (size_t)(1 + KH) * NT * sizeof(int2);
+    static_assert(D < 3 || cell_bytes <= mix_bytes, "the cells fit");
+    static size_t bytes_of(const Geo& g) { return g.mixed ? bytes : bytes - mix_bytes + (D == 3 ? cell_bytes : 0); }
 };
 // The geometry and buffers of a batch member, copied to shared memory at the
 // start of an item (a reference into the table costs a global load per use, a
@@ -312,7 +316,8 @@ __device__ __forceinline__ void end_faces(const Geo& g, const Bufs<T>& bf, int a
 // batched step runs the same body.  g and bf lie in the constant bank (single instances) or in shared
 // memory (batches) and are read where they are used, which keeps the loop's
 // registers for the chunk in flight.
-template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true>
+template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true,
+          bool AL = true>
 __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int tile, int grp, unsigned char* smem) {
     using US = USmem<T, D, T0_, T1_, T2_, TAB, SK>;
     using TL = typename US::TL;
@@ -338,7 +343,15 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
     bool valid = true;
 #pragma unroll
     for (int a = 0; a < D; ++a) valid = valid && qa[a] < g.n[a];
-    int src[1 + KH], kfl[1 + KH];                    // source cell (-1 none); box index | boundary flags << 16
+    // per cell: the source cell (-1 none), box index | boundary flags << 16
+    constexpr bool CS = D == 3 && !MIX;
+    int2 cells[CS ? 1 : 1 + KH];
+    int2* const CL = reinterpret_cast<int2*>(ring + US::RING * US::rec_bytes) + threadIdx.x;
+    auto cell = [&](int r) -> int2& {
+        if constexpr (CS) return CL[r * NT];
+        else return cells[r];
+    };
+    const int k0 = TL::box_of(la[0], la[1], la[2]);
 #pragma unroll
     for (int r = 0; r <= KH; ++r) {
         int l[3] = {la[0], la[1], la[2]};
@@ -362,8 +375,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         bool dir;
         resolve<D>(g, q, refl, dir);
         const long long c = cell_index(g, q);
-        src[r] = on ? (int)c : -1;
-        kfl[r] = TL::box_of(l[0], l[1], l[2]) | (refl | (dir ? 8 : 0)) << 16;
+        cell(r) = make_int2(on ? (int)c : -1, TL::box_of(l[0], l[1], l[2]) | (refl | (dir ? 8 : 0)) << 16);
     }
 
     if (j0 >= j1) return;
@@ -404,14 +416,15 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         }
 #pragma unroll
         for (int r = 0; r <= KH; ++r) {
-            if (src[r] < 0) continue;
-            const unsigned c = (unsigned)src[r];
-            const int f = kfl[r] >> 16;
+            const int2 cl = cell(r);
+            if (cl.x < 0) continue;
+            const unsigned c = (unsigned)cl.x;
+            const int f = cl.y >> 16;
             if (f == 0) {
                 cp_async_chunk_ca(&slot(SPH, r), row + (unsigned long long)c * N8);
                 cp_async_chunk_ca(&slot(SPH + 1, r), row + (unsigned long long)c * N8 + VC);
                 if constexpr (TAB) {
-                    if (g.xal) {
+                    if constexpr (AL) {
                         if (r0 != row0) cp_async_chunk_ca(&slot(SX0, r), px0 + (unsigned long long)c * VC);
                         x12[r][0] = __ldg(px1 + c);
                         if constexpr (D == 3) x12[r][1] = __ldg(px2 + c);
@@ -429,7 +442,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                 }
             }
             if constexpr (TAB) {
-                if (g.xal) {
+                if constexpr (AL) {
                     const T* X = (f & 8) ? bf.xc0 : bf.xc;
                     if (r0 != row0)
                         cp_async_chunk_ca(&slot(SX0, r), X + (size_t)((f & 1) ? g.nv1[0] - VC - r0 : r0) * nn + (size_t)VC * c);
@@ -452,9 +465,10 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
     }
 #pragma unroll
     for (int r = 0; r <= KH; ++r) {
-        if (src[r] < 0) continue;
-        const int refl = kfl[r] >> 16 & 7;
-        const CellC<T>& cs = (kfl[r] >> 16 & 8) ? bf.cellc0[src[r]] : bf.cellc[src[r]];
+        const int2 cl = cell(r);
+        if (cl.x < 0) continue;
+        const int refl = cl.y >> 16 & 7;
+        const CellC<T>& cs = (cl.y >> 16 & 8) ? bf.cellc0[cl.x] : bf.cellc[cl.x];
         T cst[4 * NCV];
 #pragma unroll
         for (int i = 0; i < 4 * NCV; ++i) cst[i] = T(0);
@@ -559,8 +573,9 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
             const K hx = vr[3];
 #pragma unroll
             for (int r = 0; r <= KH; ++r) {
-                if (src[r] < 0) continue;
-                const int fl = kfl[r] >> 16;
+                const int2 cl = cell(r);
+                if (cl.x < 0) continue;
+                const int fl = cl.y >> 16;
                 T cst[4 * NCV];
 #pragma unroll
                 for (int i = 0; i < NCV; ++i) {
@@ -572,7 +587,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                 constexpr int o = TAB ? 3 : D + 2, oh = TAB ? 3 : D + 3;
                 K ge, pb;
                 if constexpr (TAB) {
-                    if (g.xal) {
+                    if constexpr (AL) {
                         K x = slot(SX0, r);
                         if (fl & 1) {
                             T y[VC];
@@ -582,23 +597,27 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                         }
                         ge = x * K::bc(lean_pair<T, D>(x12[r][0], x12[r][1]));
                     } else {
-                        const T* X = (fl & 8) ? bf.xc0 : bf.xc;
-                        const size_t nn = (size_t)g.Nc;
+                        // a chunk's lanes lie in at most two velocity rows (the first
+                        // lane's and the last one's); a mirror image takes the mirrored ones
+                        const int* const ri = rec_int(j);
+                        const unsigned long long nn = (unsigned)g.Nc, c = (unsigned)cl.x;
+                        const T* const X = (fl & 8) ? bf.xc0 : bf.xc;
+                        const int m0 = g.nv1[0] - 1, m1 = 2 * g.xrow[1] + g.nv1[1] - 1, m2 = 2 * g.xrow[2] + g.nv1[2] - 1;
+                        auto row = [&](int v) {
+                            const int r1 = ri[8 + v], r2 = ri[12 + v];
+                            const T x1 = __ldg(X + (unsigned)((fl & 2) ? m1 - r1 : r1) * nn + c);
+                            return lean_pair<T, D>(x1, D == 3 ? __ldg(X + (unsigned)((fl & 4) ? m2 - r2 : r2) * nn + c) : T(1));
+                        };
+                        const int last = ri[7] < 0 ? 0 : 3;      // (padding only follows lanes of one row)
+                        const T pa = row(0);
+                        T pb = pa;
+                        if (ri[8 + last] != ri[8] || ri[12 + last] != ri[12]) pb = row(3);
                         T y[VC];
 #pragma unroll
                         for (int v = 0; v < VC; ++v) {
-                            int r0 = rec_int(j)[4 + v], r1 = rec_int(j)[8 + v];
-                            y[v] = T(0);
-                            if (r0 < 0) continue;            // padding
-                            if (fl & 1) r0 = g.nv1[0] - 1 - r0;
-                            if (fl & 2) r1 = 2 * g.xrow[1] + g.nv1[1] - 1 - r1;
-                            T z = __ldg(X + (size_t)r1 * nn + src[r]);
-                            if constexpr (D == 3) {
-                                int r2 = rec_int(j)[12 + v];
-                                if (fl & 4) r2 = 2 * g.xrow[2] + g.nv1[2] - 1 - r2;
-                                z = lean_pair<T, D>(z, __ldg(X + (size_t)r2 * nn + src[r]));
-                            }
-                            y[v] = __ldg(X + ((size_t)(r0 / VC) * nn + src[r]) * VC + (r0 % VC)) * z;
+                            const int k = ri[4 + v], k0 = (fl & 1) ? m0 - k : k;
+                            const bool in_a = ri[8 + v] == ri[8] && ri[12 + v] == ri[12];
+                            y[v] = k < 0 ? T(0) : __ldg(X + ((unsigned)(k0 / VC) * nn + c) * VC + (k0 % VC)) * (in_a ? pa : pb);
                         }
                         ge = K::of(y);
                     }
@@ -618,8 +637,8 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                         pb = fma4(K::bc(cst[o + 4]) * z, dg, pb);
                     }
                 }
-                Pg[kfl[r] & 0xffff] = pg;
-                Pb[kfl[r] & 0xffff] = pb;
+                Pg[cl.y & 0xffff] = pg;
+                Pb[cl.y & 0xffff] = pb;
             }
         }
         if (j + 1 < j1) {                            // in flight over the rest of this visit
@@ -631,11 +650,11 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         // (one barrier per visit: the other buffer is written next, and this one
         // again only after the next barrier, past which every thread has read it)
         if (valid) {
-            const int k0 = kfl[0] & 0xffff;
             K vg[D];                                 // g at the main side's faces
             T sm[D * NM];
 #pragma unroll
             for (int f = 0; f < 2; ++f) {
+                if (D == 3) asm volatile("" ::: "memory");     // b's neighbours not before g is done: registers
                 const K* const Pf = (f ? Pb : Pg) + k0;
                 const K c = Pf[0];
                 K base = c, hs[D];
@@ -713,6 +732,9 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
             }
         }
     } else {
+        int tl = tile;
+        keep(tl);                                    // (found again here rather than kept over the loop)
+        tile_origin<TL, D>(g, tl, org);
         static_assert(NM * sizeof(T) * NT <= US::bytes, "the moments of a round in shared memory");
 #pragma unroll 1
         for (int a = 0; a < D; ++a) {
@@ -727,14 +749,15 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
     }
 }
 
-// MIX = false: for instances without mixed visits (3D, where the other side's
-// values and sums would not fit the registers).
-template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true>
+// MIX = false: for instances without mixed visits, AL = false (TAB): whose
+// velocity rows are not whole chunks.  Each variant's loop holds only what it
+// needs: in 3D the registers and the loop's code size are the limit.
+template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true, bool AL = true>
 __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (UOcc<T, D, T0_, T1_, T2_, TAB, SK>::value))
     k_usweep(const __grid_constant__ Geo g, const __grid_constant__ Bufs<T> bf) {
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_wait();
-    usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, MIX>(g, bf, blockIdx.x, blockIdx.y, smem);
+    usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, MIX, AL>(g, bf, blockIdx.x, blockIdx.y, smem);
 }
 
 template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false>
@@ -746,7 +769,10 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (UOcc<T, D, T0_, T
     pdl_wait();
     const Item it = items[blockIdx.x];
     rec.load(insts[it.inst], cur[it.inst] & 1);
-    usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK>(rec.g, rec.b, it.tile, it.grp, smem);
+    if (TAB && !rec.g.xal)
+        usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, true, !TAB>(rec.g, rec.b, it.tile, it.grp, smem);
+    else
+        usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK>(rec.g, rec.b, it.tile, it.grp, smem);
 }
 
 }  // namespace cdg
