@@ -61,7 +61,7 @@ enum { BUF_PHIBAR = 1, BUF_SLOPES = 2, BUF_FACES = 4, BUF_FORCE = 8, BUF_XTAB = 
 int buffers_of(int mode) {
     int b = 0;
     if (cdg::mode_upwind(mode)) b |= BUF_VISITS;
-    if (cdg::mode_faces(mode) && !cdg::mode_acc(mode)) b |= BUF_CHUNKS;
+    if (cdg::mode_faces(mode)) b |= BUF_CHUNKS;
     if (cdg::mode_lean(mode)) b |= BUF_XTAB;
     if (cdg::mode_acc(mode)) b |= BUF_FORCE;
     if (cdg::mode_source(mode) != cdg::MODE_FUSED) b |= BUF_PHIBAR;
@@ -193,13 +193,22 @@ void build_visits(cdugks* h) {
     };
     const int n0c = g.nv1[0] / VC, m = g.nv1[1] * g.nv1[2];
     auto order = [&](int vt) { return g.xal ? (vt % n0c) * m + vt / n0c : vt; };
+    // sweep B: the same, but with an acceleration along one axis that axis's nodes
+    // fastest, so that the chunks of neighbouring nodes, which the force gradients
+    // read, follow each other (cache hits)
+    const int fa = !g.accel ? -1 : (g.acc[0] != 0.0 ? 0 : (g.acc[1] != 0.0 ? 1 : 2));
+    auto b_order = [&](int vt) {
+        if (!g.xal || fa == 0) return vt;
+        if (fa != 2) return order(vt);
+        return (vt % n0c * g.nv1[1] + vt / n0c % g.nv1[1]) * g.nv1[2] + vt / (n0c * g.nv1[1]);
+    };
     std::vector<Visit> vis, chunks;
     vis.reserve(g.NVT + 16);
     chunks.resize(g.NVT);
     for (int vt = 0; vt < g.NVT; ++vt) {
         const unsigned char* ps = &pos[(size_t)vt * VC];
         const unsigned char* zs = &zero[(size_t)vt * VC];
-        chunks[order(vt)] = Visit{0, vt, 0, 0};
+        chunks[b_order(vt)] = Visit{0, vt, 0, 0};
         unsigned seen = 0;
         for (int v = 0; v < VC; ++v) {
             const int own = ps[v] & mask;
@@ -285,7 +294,7 @@ void set_groups(cdugks* h, int G) {
     g.G = (g.NVT + g.ntpg - 1) / g.ntpg;
     for (int a = 0; a < 3; ++a) g.ws[a] = g.G;
     const int mode = tile_mode(h->prec, g.D, g.tile_id);
-    g.upw = cdg::mode_upwind(mode) && !(cdg::mode_sk(mode) && h->zero_node);
+    g.upw = cdg::mode_upwind(mode) && !((cdg::mode_sk(mode) || cdg::mode_acc(mode)) && h->zero_node);
     if (!g.upw) return;
     h->slots.assign((size_t)g.G * 6, -1);
     for (int a = 0; a < 3; ++a) g.ws[a] = 0;
@@ -788,6 +797,7 @@ int cdugks_set_acceleration(cdugks_t* h, const double* a) {
     const Geo old = h->g;
     for (int b = 0; b < 3; ++b) h->g.acc[b] = acc[b];
     h->g.accel = on;
+    build_visits(h);             // (sweep B's chunk order)
     const int rc = cdugks_set_tile(h, id);
     if (rc) h->g = old;
     return rc;

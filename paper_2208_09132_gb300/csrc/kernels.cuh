@@ -841,12 +841,13 @@ __host__ __device__ constexpr bool mode_nosrc(int mode) { return (mode & (MODE_N
 __host__ __device__ constexpr int mode_halo(int mode) { return mode_r2(mode) ? 3 : 2; }
 __host__ __device__ constexpr bool mode_lean(int mode) { return (mode & MODE_LEAN) != 0; }
 __host__ __device__ constexpr bool mode_xf(int mode) { return (mode & MODE_XF) != 0; }
-// Shapes whose sweep A is usweep.cuh's: the lean shapes and the fused
-// face-store shapes of the upwind-cell reconstruction, of either collision
-// model (the Shakhov model on velocity grids with a node at 0 keeps the fused
-// sweep: its heat flux reads the stored face values of those nodes, Geo::upw).
+// Shapes whose sweep A is usweep.cuh's: the lean shapes, and the fused and the
+// acceleration face-store shapes of the upwind-cell reconstruction (of either
+// collision model).  With the Shakhov model or the acceleration a velocity grid
+// with a node at 0 keeps the fused sweep (Geo::upw): the heat flux and the force
+// gradients read the stored face values of those nodes.
 __host__ __device__ constexpr bool mode_upwind(int mode) {
-    return mode_faces(mode) && mode_source(mode) == MODE_FUSED && !mode_r2(mode) && !mode_acc(mode);
+    return mode_faces(mode) && (mode_source(mode) == MODE_FUSED || mode_acc(mode)) && !mode_r2(mode);
 }
 
 template <typename T, int D, int T0, int T1, int T2, int MODE = MODE_FUSED>
@@ -2177,247 +2178,6 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (Occ<T, D, T0_, T1
     sweep_body<T, D, T0_, T1_, T2_, SWEEP_B, MODE>(in->g, in->b[cur], blockIdx.x, blockIdx.y, smem, &tm);
 }
 
-// ---- sweep B of the face-store shapes
-//
-// One CTA per (tile, velocity group), one thread per owned cell, the tiling
-// of the sweeps.  Per chunk each thread reads the stored values of both faces
-// of its cell along every axis, forms their fluxes and phi* of its cell from
-// the net flux.  A face shared by two cells is formed by both, from the same
-// values with the same arithmetic, so both see the same flux; there is no
-// exchange between threads and no barrier inside the chunk loop.  A face's
-// moments are summed by its owner (the cell on its right; the last cell for
-// the domain's right end), in chunk order.
-
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK = false>
-struct FluxSmem {
-    using TL = Tile<D, T0_, T1_, T2_>;
-    static constexpr int NPL = TL::NPL;
-    __host__ __device__ static constexpr int plane(int a) { return TL::plane(a); }
-    __host__ __device__ static constexpr int poff(int a) { return TL::poff(a); }
-    static_assert(TL::poff(D) == TL::NPL, "one slot per cell of each tile face");
-    static constexpr size_t nV4 = (size_t)FacePack<D, SK>::NV * TL::NFT;
-    static constexpr size_t bytes = nV4 * sizeof(V4<T>) + (size_t)NPL * (2 + D) * sizeof(Kahan<T>);
-};
-
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK = false, bool ACC = false, bool NOSRC = false,
-          bool PERS = false>
-__device__ __forceinline__ void flux_body(const Geo g, const Bufs<T> bf, int tile, int grp, unsigned char* smem) {
-    constexpr bool NC = !PERS;      // the persistent batched step reads coherently
-    using TL = Tile<D, T0_, T1_, T2_>;
-    using FS = FluxSmem<T, D, T0_, T1_, T2_, SK>;
-    using Q = V4<T>;
-    constexpr int NM = 2 + D, NFT = TL::NFT, NFCV = FacePack<D, SK>::NV;
-    Q* const FC = reinterpret_cast<Q*>(smem);     // [NFCV][NFT] packed face constants
-    // running sums of the faces at the domain's right end, [NM][plane cell] per axis
-    Kahan<T>* const RS = reinterpret_cast<Kahan<T>*>(smem + FS::nV4 * sizeof(Q));
-    const int t = threadIdx.x;
-    int org[3];
-    tile_origin<TL, D>(g, tile, org);
-    const int vt0 = grp * g.ntpg, vt1 = min(g.NVT, vt0 + g.ntpg);
-    const int la[3] = {t % TL::T0, D >= 2 ? (t / TL::T0) % TL::T1 : 0, D >= 3 ? t / (TL::T0 * TL::T1) : 0};
-    const int qa[3] = {org[0] + la[0], org[1] + la[1], org[2] + la[2]};
-    bool valid = true;
-#pragma unroll
-    for (int a = 0; a < D; ++a) valid = valid && qa[a] < g.n[a];
-    stage_face_consts<T, D, TL, SK>(g, bf, org, FC);
-    for (int k = t; k < FS::NPL * NM; k += TL::NT) RS[k].zero();
-    __syncthreads();
-    if (!valid) return;          // no barrier below
-
-    const CellC<T> own = bf.cellc[cell_index(g, qa)];
-    const T hL = (T)(0.5 * (3.0 - D + g.K));
-    const T dtT = (T)g.dt;                        // converted once, outside the chunk loop
-    const T idxT[3] = {(T)g.idx[0], (T)g.idx[1], (T)g.idx[2]};
-    const size_t cell_ad = phi_addr(g, cell_index(g, qa), 0, 0);
-    const size_t chunk_stride = (size_t)g.Nc * (2 * VC);
-    bool own_right[3] = {false, false, false};
-    int ff[3];                   // global left face per axis (the right one is ff + face stride; < 2^31)
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        own_right[a] = qa[a] == g.n[a] - 1;
-        ff[a] = (int)face_index(g, a, qa);
-    }
-    Kahan<T> acc[D][NM];         // the left faces
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-#pragma unroll
-        for (int m = 0; m < NM; ++m) acc[a][m].zero();
-    // The first thread of each x-row of the tile asks L2 for the row's data of
-    // the next chunk while this one is formed: its cells' phi*, its left faces
-    // along every axis (along x the row's right end too), and along y / z the
-    // faces above the tile's last row.  Rows are contiguous in every layout.
-    // (Not with the force terms, whose reads of neighbouring velocity chunks
-    // measured slower with it.)
-    const bool row_lead = !ACC && la[0] == 0;
-    const int nrow = min(TL::T0, g.n[0] - org[0]);
-    constexpr int RB = 2 * VC * (int)sizeof(T);     // bytes per cell or face and chunk
-    const int tdim[3] = {TL::T0, TL::T1, TL::T2};
-
-    for (int vt = vt0; vt < vt1; ++vt) {
-        if (row_lead && vt + 1 < vt1) {
-            prefetch_l2(bf.phi_in + cell_ad + (size_t)(vt + 1) * chunk_stride, nrow * RB);
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                const T* fb = bf.face[a] + face_addr(g, a, ff[a], vt + 1);
-                prefetch_l2(fb, (nrow + (a == 0 ? 1 : 0)) * RB);
-                if (a > 0 && (la[a] == tdim[a] - 1 || own_right[a])) {
-                    const int fs = a == 1 ? g.fn[1][0] : g.fn[2][0] * g.fn[2][1];
-                    prefetch_l2(fb + (size_t)fs * (2 * VC), nrow * RB);
-                }
-            }
-        }
-        T xi[VC][D], w[VC], hx[VC];
-#pragma unroll
-        for (int v = 0; v < VC; ++v) {
-            const Q* rec = reinterpret_cast<const Q*>(bf.vel + (size_t)(vt * VC + v) * 8);
-            const Q r0 = rec[0];
-#pragma unroll
-            for (int a = 0; a < D; ++a) xi[v][a] = r0.v[a];
-            w[v] = r0.v[3];
-            hx[v] = rec[1].v[0];
-        }
-        const size_t ad = cell_ad + (size_t)vt * chunk_stride;
-        T gs[VC], bs[VC];
-        Chunk<T>::template load<NC>(bf.phi_in + ad, gs);
-        Chunk<T>::template load<NC>(bf.phi_in + ad + VC, bs);
-        T dFg[VC], dFb[VC];
-#pragma unroll
-        for (int v = 0; v < VC; ++v) dFg[v] = dFb[v] = T(0);
-#pragma unroll
-        for (int a = 0; a < D; ++a) {
-            Q F[2][2];           // [side][g|b]
-#pragma unroll
-            for (int side = 0; side < 2; ++side) {
-                // the right face of axis a is the left face of the next cell along a
-                const int fs = a == 0 ? 1 : (a == 1 ? g.fn[1][0] : g.fn[2][0] * g.fn[2][1]);
-                const T* src = bf.face[a] + face_addr(g, a, ff[a] + side * fs, vt);
-                T gb[VC], bb[VC];
-                Chunk<T>::template load<NC>(src, gb);
-                Chunk<T>::template load<NC>(src + VC, bb);
-                const int fl = TL::face_local(a, la[0] + (a == 0 ? side : 0), la[1] + (a == 1 ? side : 0),
-                                              la[2] + (a == 2 ? side : 0));
-                T fcst[4 * NFCV];
-#pragma unroll
-                for (int j = 0; j < NFCV; ++j) {
-                    const Q qv = FC[j * NFT + fl];
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) fcst[4 * j + e] = qv.v[e];
-                }
-                T sm[NM];
-#pragma unroll
-                for (int m = 0; m < NM; ++m) sm[m] = T(0);
-                if constexpr (ACC) {
-                    // the force at this face (a specular wall takes the normal component),
-                    // its gradients from the face values at the neighbouring velocities
-                    double fac[3] = {g.acc[0], g.acc[1], g.acc[2]};
-                    if ((side == 0 && qa[a] == 0 && g.bc[a][0] == BC_SPECULAR) ||
-                        (side == 1 && own_right[a] && g.bc[a][1] == BC_SPECULAR))
-                        fac[a] = 0.0;
-                    const long long fidx = (long long)ff[a] + side * fs;
-                    const T* fbase = bf.face[a];
-                    auto val = [&](int j, T& gv, T& bv) {
-                        const size_t fa0 = face_addr(g, a, fidx, j / VC) + (j % VC);
-                        gv = fbase[fa0];
-                        bv = fbase[fa0 + VC];
-                    };
-                    T fgg[VC], fgb[VC], axi[VC];
-                    if (g.nv1[0] % VC == 0) {        // velocity rows are whole chunks: vector loads
-                        auto chunk = [&](int vn, T (&gv)[VC], T (&bv)[VC]) {
-                            const T* p = fbase + face_addr(g, a, fidx, vn);
-                            Chunk<T>::template load<NC>(p, gv);
-                            Chunk<T>::template load<NC>(p + VC, bv);
-                        };
-                        force_gradient_chunk<T, D>(g, fac, vt, chunk, gb, bb, fgg, fgb);
-                    }
-#pragma unroll
-                    for (int v = 0; v < VC; ++v) {
-                        const int i = vt * VC + v;
-                        if (g.nv1[0] % VC != 0) {
-                            fgg[v] = fgb[v] = T(0);
-                            if (i < g.nv1[0] * g.nv1[1] * g.nv1[2])
-                                force_gradient<T, D>(g, fac, i, val, fgg[v], fgb[v]);
-                        }
-                        axi[v] = T(0);
-#pragma unroll
-                        for (int b = 0; b < D; ++b) axi[v] = fma((T)fac[b], xi[v][b], axi[v]);
-                    }
-                    face_flux<T, D, SK, true, NOSRC>(fcst, xi, w, hx, a, gb, bb, F[side][0], F[side][1], sm, hL, fgg,
-                                                     fgb, axi, (T)(0.5 * g.h));
-                } else {
-                    face_flux<T, D, SK, false, NOSRC>(fcst, xi, w, hx, a, gb, bb, F[side][0], F[side][1], sm, hL);
-                }
-                if (side == 0) {
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) acc[a][m].add(sm[m]);
-                } else if (own_right[a]) {
-                    const int pl = FS::poff(a) * NM + TL::plane_pos(a, la);
-#pragma unroll
-                    for (int m = 0; m < NM; ++m) {
-                        Kahan<T> k = RS[pl + m * FS::plane(a)];
-                        k.add(sm[m]);
-                        RS[pl + m * FS::plane(a)] = k;
-                    }
-                }
-            }
-            const T idx = idxT[a];
-#pragma unroll
-            for (int v = 0; v < VC; ++v) {
-                dFg[v] = fma(idx, F[1][0].v[v] - F[0][0].v[v], dFg[v]);
-                dFb[v] = fma(idx, F[1][1].v[v] - F[0][1].v[v], dFb[v]);
-            }
-        }
-        if constexpr (ACC) {     // + dt F^n of the own cell (eq. phiupdate's source, rectangle rule)
-            T fgo[VC], fbo[VC];
-            Chunk<T>::template load<NC>(bf.force + ad, fgo);
-            Chunk<T>::template load<NC>(bf.force + ad + VC, fbo);
-#pragma unroll
-            for (int v = 0; v < VC; ++v) {
-                dFg[v] -= fgo[v];
-                dFb[v] -= fbo[v];
-            }
-        }
-        T og[VC], ob[VC], oge[VC], obe[VC];
-        own_state<T, D, SK>(own, xi, hx, gs, bs, og, ob, oge, obe, hL);
-        T u[D];
-#pragma unroll
-        for (int a = 0; a < D; ++a) u[a] = own.u[a];
-        store_phi_star<T, D, SK || NOSRC>(dtT, xi, u, own.hu2, own.um_g, own.um_b, own.usrc, og, ob, oge, obe, dFg,
-                                          dFb, bf.phi_out + ad);
-    }
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-#pragma unroll
-        for (int m = 0; m < NM; ++m) bf.mf[a][((size_t)grp * NM + m) * g.nf[a] + ff[a]] = acc[a][m].value();
-        if (own_right[a]) {
-            const int fs = a == 0 ? 1 : (a == 1 ? g.fn[1][0] : g.fn[2][0] * g.fn[2][1]);
-            const int pl = FS::poff(a) * NM + TL::plane_pos(a, la);
-#pragma unroll
-            for (int m = 0; m < NM; ++m)
-                bf.mf[a][((size_t)grp * NM + m) * g.nf[a] + ff[a] + fs] = RS[pl + m * FS::plane(a)].value();
-        }
-    }
-}
-
-// CTAs per SM for k_flux: shared memory and threads, keeping >= 80 registers.
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK = false>
-struct FluxOcc {
-    static constexpr size_t per = FluxSmem<T, D, T0_, T1_, T2_, SK>::bytes + 1024;
-    static constexpr int by_smem = (int)((228 * 1024) / per);
-    static constexpr int by_threads = 2048 / Tile<D, T0_, T1_, T2_>::NT;
-    static constexpr int by_regs = 65536 / (Tile<D, T0_, T1_, T2_>::NT * 128);
-    static constexpr int v1 = by_smem < by_threads ? by_smem : by_threads;
-    static constexpr int v0 = v1 < by_regs ? v1 : by_regs;
-    static constexpr int value = v0 < 1 ? 1 : (v0 > 8 ? 8 : v0);
-};
-
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK = false, bool ACC = false, bool NOSRC = false>
-__global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (FluxOcc<T, D, T0_, T1_, T2_, SK>::value))
-    k_flux(const Inst<T>* __restrict__ in, int cur) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    pdl_wait();
-    flux_body<T, D, T0_, T1_, T2_, SK, ACC, NOSRC>(in->g, in->b[cur], blockIdx.x, blockIdx.y, smem);
-}
-
 // Many instances in one launch: the device table of instances and a work list
 // of items, one per CTA.  The current parity of each instance lives on the
 // device and the W-update kernel flips it, so a captured graph replays.
@@ -2430,16 +2190,6 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (Occ<T, D, T0_, T1
     const Item it = items[blockIdx.x];
     const Inst<T>& in = insts[it.inst];
     sweep_body<T, D, T0_, T1_, T2_, SWEEP_B, MODE>(in.g, in.b[cur[it.inst] & 1], it.tile, it.grp, smem);
-}
-
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK = false, bool ACC = false>
-__global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (FluxOcc<T, D, T0_, T1_, T2_, SK>::value))
-    k_flux_batch(const Item* __restrict__ items, const Inst<T>* __restrict__ insts, const int* __restrict__ cur) {
-    extern __shared__ __align__(128) unsigned char smem[];
-    pdl_wait();
-    const Item it = items[blockIdx.x];
-    const Inst<T>& in = insts[it.inst];
-    flux_body<T, D, T0_, T1_, T2_, SK, ACC>(in.g, in.b[cur[it.inst] & 1], it.tile, it.grp, smem);
 }
 
 // ---- Shakhov model: raw velocity moments for the heat flux

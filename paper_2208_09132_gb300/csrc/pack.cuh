@@ -231,7 +231,8 @@ __device__ __forceinline__ Pk<T> expo4(const Pk<T>& x) {
 // FP64 in one dimension (the FP64 pipe is the bound, and the exponential most
 // of it): the four Maxwellian values of a chunk follow from the first two by
 // the recurrence of equally spaced nodes, E_{k+1} = E_k r_k, r_{k+1} = r_k q,
-// q = exp(2 cexp dxi^2) a constant of the place -- two exponentials instead of
+// q = exp(2 cexp dxi^2) a constant of the place, kept as q - 1 (its rounding, the
+// same in every chunk, then counts |q - 1| times) -- two exponentials instead of
 // four and a handful of roundings -- unless the first one is near underflow.
 template <typename T, int D>
 __host__ __device__ constexpr bool gauss_ratio() {
@@ -239,9 +240,9 @@ __host__ __device__ constexpr bool gauss_ratio() {
 }
 template <typename T>
 __device__ __forceinline__ T gauss_q(T cexp, T dxi) {
-    return Num<T>::expo(Ar<T>::mul(T(2) * cexp, Ar<T>::mul(dxi, dxi)));
+    return (T)expm1((double)Ar<T>::mul(T(2) * cexp, Ar<T>::mul(dxi, dxi)));
 }
-__device__ __forceinline__ Pk<double> gauss_chunk(double cexp, double u, double q, double dxi, const Pk<double>& xi) {
+__device__ __forceinline__ Pk<double> gauss_chunk(double cexp, double u, double q /* - 1 */, double dxi, const Pk<double>& xi) {
     const double d0 = __dsub_rn(xi.v[0], u);
     const double e0 = exp(__dmul_rn(cexp, __dmul_rn(d0, d0)));
     Pk<double> r;
@@ -251,7 +252,7 @@ __device__ __forceinline__ Pk<double> gauss_chunk(double cexp, double u, double 
 #pragma unroll
         for (int i = 1; i < VC; ++i) {
             r.v[i] = __dmul_rn(r.v[i - 1], f);
-            f = __dmul_rn(f, q);
+            f = __fma_rn(f, q, f);
         }
     } else {
 #pragma unroll
@@ -266,7 +267,7 @@ __device__ __forceinline__ Pk<float> gauss_chunk(float, float, float, float, con
 
 // The equilibria of a chunk's velocities xi (hx = |xi|^2 / 2) at a place with
 // the constants c: u (D), cexp, pref, eb, hu2, three more, with SK sq (D) and
-// e2, with gauss_ratio q.  hL as in shakhov_point, dxi the axis-0 spacing.
+// e2, with gauss_ratio q - 1.  hL as in shakhov_point, dxi the axis-0 spacing.
 template <typename T, int D, bool SK>
 __device__ __forceinline__ void eq4(const T* c, const Pk<T>* xi, const Pk<T>& hx, T hL, T dxi, Pk<T>& ge, Pk<T>& be) {
     using K = Pk<T>;

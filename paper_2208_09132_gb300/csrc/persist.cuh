@@ -142,7 +142,7 @@ __global__ void __launch_bounds__(Tile<D, TX, TY, TZ>::NT, (PersistSmem<T, D, TX
             for (long long k = t; k < it.count; k += NT) facec_body<T, D>(in.g, in.b[c], it.a, it.start + k);
         } else if (it.kind == PK_B) {
             rec.load(in, c);
-            bflux_body<T, D, TX, TY, TZ, false, false, false, true>(rec.g, rec.b, it.a, it.b, smem);
+            bflux_body<T, D, TX, TY, TZ, false, false, false, false, true>(rec.g, rec.b, it.a, it.b, smem);
         } else {
             for (long long k = t; k < it.count; k += NT) wupdate_body<T, D>(in.g, in.b[c], it.start + k);
         }

@@ -93,12 +93,12 @@ TmaPair make_tma(const Geo& g, const void* phi_in) {
 // stored shapes (MODE_STORED) form phibar+ and the slopes (k_shslope); the
 // sweeps of both load what was formed instead of recomputing it on the halo.
 // Face-store shapes (MODE_FACES bit) have sweep A keep the reconstructed
-// face values and run k_flux as sweep B.  Shakhov shapes (MODE_SK, face-store
+// face values and run k_bflux as sweep B.  Shakhov shapes (MODE_SK, face-store
 // only) add k_faceq before the face constants and k_cellq before the W update.
 // Acceleration shapes (MODE_ACC, prepared face-store only) form the force
-// terms in k_prep and take them in k_flux.
+// terms in k_prep and take them in k_bflux.
 // Sweep B on tiles of BX x BY x BZ cells, for one instance or (BATCH) a list of items.
-template <typename T, int D, int BX, int BY, int BZ, bool SK, bool XF, bool BATCH>
+template <typename T, int D, int BX, int BY, int BZ, bool SK, bool XF, bool BATCH, bool ACC = false>
 struct BLaunch {
     using BS = BSmem<T, D, BX, BY, BZ, SK, XF>;
     using TL = typename BS::TL;
@@ -106,17 +106,17 @@ struct BLaunch {
         const auto size = [](auto* kern) {
             return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)BS::bytes);
         };
-        cudaError_t e = size(k_bflux<T, D, BX, BY, BZ, SK, true, XF>);
+        cudaError_t e = size(k_bflux<T, D, BX, BY, BZ, SK, true, XF, ACC>);
         if constexpr (!SK) {
-            if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, false, XF>);
+            if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, false, XF, ACC>);
         }
         if constexpr (BATCH) {
-            if (!e) e = size(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF>);
+            if (!e) e = size(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF, ACC>);
         }
         return e;
     }
     static cudaError_t launch_batch(const Item* items, int n, const Inst<T>* insts, const int* cur, cudaStream_t s) {
-        return launch_pdl(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF>, dim3(n), dim3(TL::NT), BS::bytes, s, items, insts, cur);
+        return launch_pdl(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF, ACC>, dim3(n), dim3(TL::NT), BS::bytes, s, items, insts, cur);
     }
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
     static cudaError_t launch(const Geo& g, const Bufs<T>& hb, cudaStream_t s) {
@@ -125,9 +125,9 @@ struct BLaunch {
         const dim3 grid(tiles, g.G);
         if constexpr (!SK) {
             if (!g.nosrc)
-                return launch_pdl(k_bflux<T, D, BX, BY, BZ, false, false, XF>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
+                return launch_pdl(k_bflux<T, D, BX, BY, BZ, false, false, XF, ACC>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
         }
-        return launch_pdl(k_bflux<T, D, BX, BY, BZ, SK, true, XF>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
+        return launch_pdl(k_bflux<T, D, BX, BY, BZ, SK, true, XF, ACC>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
     }
 };
 // The tile of sweep B (outside the persistent step, whose blocks are those of
@@ -166,7 +166,6 @@ template <typename T, int D, int TX, int TY, int TZ, int MODE = MODE_FUSED, bool
 struct Shape {
     static constexpr bool SK = mode_sk(MODE);
     using SM = Smem<T, D, TX, TY, TZ, MODE>;
-    using FS = FluxSmem<T, D, TX, TY, TZ, SK>;
     using TL = Tile<D, TX, TY, TZ>;
     static constexpr int mode = MODE;
     static constexpr int SRC = mode_source(MODE);
@@ -184,17 +183,18 @@ struct Shape {
     // shapes (their pre-pass is batched too)
     static constexpr bool BATCH = SRC == MODE_FUSED || ACC;
     using BT = BTile<T, D, TX, TY, TZ>;
-    using BL = BLaunch<T, D, BT::X, BT::Y, BT::Z, SK, false, BATCH>;
+    using BL = BLaunch<T, D, BT::X, BT::Y, BT::Z, SK, false, BATCH, ACC>;
     // sweep A with upwind owners (usweep.cuh)
     static constexpr bool UP = mode_upwind(MODE);
     using US = USmem<T, D, TX, TY, TZ, false, SK>;
-    // sweep B of the face-store shapes: bflux.cuh's, or k_flux with the acceleration
-    static constexpr bool BF = FACES && !ACC;
+    // (Shakhov and acceleration shapes keep the fused or prepared sweep too, for
+    // velocity grids with a node at 0: Geo::upw)
+    static constexpr bool OLD_A = !UP || SK || ACC;
 
     // dynamic shared memory of the larger of the two sweeps
     static size_t smem_bytes() {
         const size_t a = UP ? US::bytes : SM::bytes(false);
-        const size_t b = BF ? BL::BS::bytes : (FACES ? FS::bytes : SM::bytes(true));
+        const size_t b = FACES ? BL::BS::bytes : SM::bytes(true);
         return a > b ? a : b;
     }
 
@@ -205,12 +205,8 @@ struct Shape {
         if ((e = cudaFuncSetAttribute(k_sweep<T, D, TX, TY, TZ, false, MODE>,
                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
             return e;
-        if constexpr (BF) {
+        if constexpr (FACES) {
             if ((e = BL::configure())) return e;
-        } else if constexpr (FACES) {
-            if ((e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, SK, ACC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)FS::bytes)))
-                return e;
         } else {
             if ((e = cudaFuncSetAttribute(k_sweep<T, D, TX, TY, TZ, true, MODE>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(true))))
@@ -220,20 +216,15 @@ struct Shape {
             const auto size = [](auto* kern) {
                 return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)US::bytes);
             };
-            if ((e = size(k_usweep<T, D, TX, TY, TZ, false, true, SK>)) ||
-                (e = size(k_usweep_batch<T, D, TX, TY, TZ, false, SK, SK>)))
+            if ((e = size(k_usweep<T, D, TX, TY, TZ, false, true, SK, true, true, ACC>)) ||
+                (e = size(k_usweep_batch<T, D, TX, TY, TZ, false, SK || ACC, SK, ACC>)))
                 return e;
-            if constexpr (NS) {
+            if constexpr (NS && !ACC) {
                 if ((e = size(k_usweep<T, D, TX, TY, TZ, false, false>))) return e;
             }
         } else if constexpr (NS) {
             if ((e = cudaFuncSetAttribute(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>,
                                           cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
-                return e;
-        }
-        if constexpr (NS && ACC) {
-            if ((e = cudaFuncSetAttribute(k_flux<T, D, TX, TY, TZ, false, ACC, true>,
-                                          cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)))
                 return e;
         }
         if constexpr (SRC == MODE_STORED) {
@@ -242,16 +233,12 @@ struct Shape {
                 return e;
         }
         if constexpr (BATCH) {
-            if constexpr (!UP || SK) {
+            if constexpr (OLD_A) {
                 if ((e = cudaFuncSetAttribute(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(false))))
                     return e;
             }
-            if constexpr (FACES && !BF) {
-                if ((e = cudaFuncSetAttribute(k_flux_batch<T, D, TX, TY, TZ, SK, ACC>,
-                                              cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FS::bytes)))
-                    return e;
-            } else if constexpr (!FACES) {
+            if constexpr (!FACES) {
                 if ((e = cudaFuncSetAttribute(k_sweep_batch<T, D, TX, TY, TZ, true, MODE>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SM::bytes(true))))
                     return e;
@@ -267,7 +254,14 @@ struct Shape {
         if (e) return e;
         const dim3 grid(g.tiles[0] * g.tiles[1] * g.tiles[2], g.G);
         if (ev) cudaEventRecord(ev[0], s);
-        if constexpr (SRC == MODE_PREP) {
+        const int ax = !ACC ? -1 : (g.acc[0] != 0.0 ? 0 : (g.acc[1] != 0.0 ? 1 : 2));
+        const int axes = (g.acc[0] != 0.0) + (g.acc[1] != 0.0) + (g.acc[2] != 0.0);
+        const int len = ax == 0 ? g.nv1[0] / VC : (ax > 0 ? g.nv1[ax] : 1);
+        if (ACC && g.xal && axes == 1 && g.NVT / len < 65536) {    // a line of the forced axis's chunks per block row
+            const dim3 lg((unsigned)((g.Nc + kPrepCells - 1) / kPrepCells), (unsigned)(g.NVT / len));
+            if constexpr (ACC) e = launch_pdl(k_prep_line<T, D>, lg, dim3(kPrepCells), 0, s, g, hb, ax, len);
+            if (e) return e;
+        } else if constexpr (SRC == MODE_PREP) {
             const dim3 pg((unsigned)((g.Nc + kPrepCells - 1) / kPrepCells),
                           (unsigned)((g.NVT + kPrepChunks - 1) / kPrepChunks));
             if ((e = launch_pdl(k_prep<T, D, ACC>, pg, dim3(kPrepCells), 0, s, in, cur, kPrepChunks))) return e;
@@ -278,13 +272,14 @@ struct Shape {
         }
         const bool ns = NS && g.nosrc, up = UP && g.upw && !g.wait_test;
         if constexpr (UP) {
-            if (up && (ns || SK)) {
-                e = launch_pdl(k_usweep<T, D, TX, TY, TZ, false, true, SK>, grid, dim3(TL::NT), US::bytes_of(g), s, g, hb);
+            const auto a = [&](auto* kern) { return launch_pdl(kern, grid, dim3(TL::NT), US::bytes_of(g), s, g, hb); };
+            if constexpr (SK || ACC) {
+                if (up) e = a(k_usweep<T, D, TX, TY, TZ, false, true, SK, true, true, ACC>);
             } else if (up) {
-                if constexpr (NS) e = launch_pdl(k_usweep<T, D, TX, TY, TZ, false, false>, grid, dim3(TL::NT), US::bytes_of(g), s, g, hb);
+                e = ns ? a(k_usweep<T, D, TX, TY, TZ, false, true>) : a(k_usweep<T, D, TX, TY, TZ, false, false>);
             }
         }
-        if (!up) {      // (a shape with upwind owners: the Shakhov model with a node at 0, and the wait hook)
+        if (!up) {      // (a shape with upwind owners: a node at 0, see OLD_A, and the wait hook)
             const TmaPair tma = make_tma<T, D, typename SM::TL>(g, SM::stage(false) ? phi_in : nullptr);
             if constexpr (NS && !UP) {
                 if (ns)
@@ -309,13 +304,7 @@ struct Shape {
             if ((e = launch_pdl(k_facec<T, D>, fgrid, dim3(kSmallBlock), 0, s, in, cur))) return e;
         }
         if (ev) cudaEventRecord(ev[2], s);
-        if constexpr (BF) {
-            e = BL::launch(g, hb, s);
-        } else if constexpr (NS) {
-            if (ns) e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, ACC, true>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
-            else e = launch_pdl(k_flux<T, D, TX, TY, TZ, false, ACC>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
-        } else if constexpr (FACES)
-            e = launch_pdl(k_flux<T, D, TX, TY, TZ, SK, ACC>, grid, dim3(TL::NT), FS::bytes, s, in, cur);
+        if constexpr (FACES) e = BL::launch(g, hb, s);
         else e = launch_pdl(k_sweep<T, D, TX, TY, TZ, true, MODE>, grid, dim3(TL::NT), SM::bytes(true), s, in, cur,
                             make_tma<T, D, TL>(g, nullptr));
         if (e) return e;
@@ -342,19 +331,16 @@ struct Shape {
             if (!B) {
                 if constexpr (UP) {
                     if (up)
-                        return launch_pdl(k_usweep_batch<T, D, TX, TY, TZ, false, SK, SK>, dim3(n), dim3(TL::NT), US::bytes,
-                                          s, items, insts, cur);
+                        return launch_pdl(k_usweep_batch<T, D, TX, TY, TZ, false, SK || ACC, SK, ACC>, dim3(n), dim3(TL::NT),
+                                          US::bytes, s, items, insts, cur);
                 }
-                if constexpr (!UP || SK)
+                if constexpr (OLD_A)
                     return launch_pdl(k_sweep_batch<T, D, TX, TY, TZ, false, MODE>, dim3(n), dim3(TL::NT),
                                       SM::bytes(false), s, items, insts, cur);
                 return cudaErrorNotSupported;
             }
-            if constexpr (BF)
+            if constexpr (FACES)
                 return BL::launch_batch(items, n, insts, cur, s);
-            else if constexpr (FACES)
-                return launch_pdl(k_flux_batch<T, D, TX, TY, TZ, SK, ACC>, dim3(n), dim3(TL::NT), FS::bytes, s, items,
-                                  insts, cur);
             else
                 return launch_pdl(k_sweep_batch<T, D, TX, TY, TZ, true, MODE>, dim3(n), dim3(TL::NT), SM::bytes(true), s,
                                   items, insts, cur);
@@ -363,7 +349,7 @@ struct Shape {
 
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
     static TileShape b_shape() {
-        if constexpr (BF) return BL::shape();
+        if constexpr (FACES) return BL::shape();
         else return shape();
     }
     static int a_ctas() {
@@ -396,7 +382,7 @@ struct Shape {
 };
 
 // A lean shape (lean.cuh): sweep A k_usweep, face constants (with the face
-// factor tables when XF), sweep B k_lflux (XF) or k_flux, W update (with the
+// factor tables when XF), sweep B k_bflux (equilibria from them with XF), W update (with the
 // cell factor tables).  Single instances take the sweeps without the b-source
 // terms when the instance has none (Pr = 1); batched launches keep the general
 // ones.

@@ -105,7 +105,7 @@ struct UOcc {
 
 // phibar+ of the cell with coordinates q (ghosts included) for the four
 // velocities of one chunk, straight from global memory (end cells only).
-template <typename T, int D, bool TAB, bool NOSRC, bool SK>
+template <typename T, int D, bool TAB, bool NOSRC, bool SK, bool PRE>
 __device__ __noinline__ void phibar_at(const Geo& g, const Bufs<T>& bf, int q0, int q1, int q2, int vt,
                                           const T* __restrict__ vr, T (&pg)[VC], T (&pb)[VC]) {
     int q[3] = {q0, q1, q2};
@@ -113,6 +113,15 @@ __device__ __noinline__ void phibar_at(const Geo& g, const Bufs<T>& bf, int q0, 
     bool dir;
     resolve<D>(g, q, refl, dir);
     const long long c = cell_index(g, q);
+    if (PRE && !dir) {             // formed by the pre-pass
+#pragma unroll
+        for (int v = 0; v < VC; ++v) {
+            const int i = vt * VC + v, is = refl ? bf.refl[refl * g.Nvp + i] : i;
+            pg[v] = bf.phibar[phi_addr(g, c, is, 0)];
+            pb[v] = bf.phibar[phi_addr(g, c, is, 1)];
+        }
+        return;
+    }
     const CellC<T>& cs = dir ? bf.cellc0[c] : bf.cellc[c];
     T u[D];
 #pragma unroll
@@ -172,7 +181,7 @@ __device__ __noinline__ void phibar_at(const Geo& g, const Bufs<T>& bf, int q0, 
 // one (end cell, visit) pair per thread and round; the end cells' threads add
 // the visits' moments in order.  Not inlined: kept out of the sweep's registers
 // and code.
-template <typename T, int D, typename TL, bool TAB, bool NOSRC, bool SK>
+template <typename T, int D, typename TL, bool TAB, bool NOSRC, bool SK, bool PRE>
 __device__ __noinline__ void edge_pass(const Geo& g, const Bufs<T>& bf, int org0, int org1, int org2, int a, int side, int j0,
                                        int j1, int slot, T* red) {
     constexpr int NM = 2 + D, NT = TL::NT;
@@ -205,7 +214,7 @@ __device__ __noinline__ void edge_pass(const Geo& g, const Bufs<T>& bf, int org0
             const int vt = __ldg(bf.vint + (size_t)kVisitInts * j);
             const T* vr = bf.vrec + (size_t)j * (kVisitVecs * VC);
             T base[2][VC], ctr[2][VC], hsa[2][VC];
-            phibar_at<T, D, TAB, NOSRC, SK>(g, bf, q[0], q[1], q[2], vt, vr, base[0], base[1]);
+            phibar_at<T, D, TAB, NOSRC, SK, PRE>(g, bf, q[0], q[1], q[2], vt, vr, base[0], base[1]);
 #pragma unroll
             for (int v = 0; v < VC; ++v) {
                 ctr[0][v] = base[0][v];
@@ -214,8 +223,8 @@ __device__ __noinline__ void edge_pass(const Geo& g, const Bufs<T>& bf, int org0
 #pragma unroll 1
             for (int e = 0; e < D; ++e) {
                 T lo[2][VC], hi[2][VC];
-                phibar_at<T, D, TAB, NOSRC, SK>(g, bf, q[0] - (e == 0), q[1] - (e == 1), q[2] - (e == 2), vt, vr, lo[0], lo[1]);
-                phibar_at<T, D, TAB, NOSRC, SK>(g, bf, q[0] + (e == 0), q[1] + (e == 1), q[2] + (e == 2), vt, vr, hi[0], hi[1]);
+                phibar_at<T, D, TAB, NOSRC, SK, PRE>(g, bf, q[0] - (e == 0), q[1] - (e == 1), q[2] - (e == 2), vt, vr, lo[0], lo[1]);
+                phibar_at<T, D, TAB, NOSRC, SK, PRE>(g, bf, q[0] + (e == 0), q[1] + (e == 1), q[2] + (e == 2), vt, vr, hi[0], hi[1]);
 #pragma unroll
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
@@ -311,13 +320,14 @@ __device__ __forceinline__ void end_faces(const Geo& g, const Bufs<T>& bf, int a
 }
 
 // TAB: equilibria from the cell factor tables (lean shapes), else one
-// exponential per point (SK: with the Shakhov correction).  What other kernels
+// exponential per point (SK: with the Shakhov correction); PRE: phibar+ from the
+// pre-pass (acceleration).  What other kernels
 // or items wrote is read through coherent copies and loads, so the persistent
 // batched step runs the same body.  g and bf lie in the constant bank (single instances) or in shared
 // memory (batches) and are read where they are used, which keeps the loop's
 // registers for the chunk in flight.
 template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true,
-          bool AL = true>
+          bool AL = true, bool PRE = false>
 __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int tile, int grp, unsigned char* smem) {
     using US = USmem<T, D, T0_, T1_, T2_, TAB, SK>;
     using TL = typename US::TL;
@@ -407,7 +417,8 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         const int4 vi = *reinterpret_cast<const int4*>(ri);       // chunk, flags, rows of axes 1 and 2
         const int vt = vi.x, r0 = TAB ? ri[4] : 0;
         const unsigned long long nn = (unsigned)g.Nc;
-        const T* const row = bf.phi_in + (unsigned)vt * (nn * N8);
+        const T* const phi = PRE ? bf.phibar : bf.phi_in;
+        const T* const row = phi + (unsigned)vt * (nn * N8);
         const T *px0 = nullptr, *px1 = nullptr, *px2 = nullptr;
         if constexpr (TAB) {
             px0 = bf.xc + (unsigned)r0 * nn;
@@ -436,7 +447,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
 #pragma unroll
                 for (int v = 0; v < VC; ++v) {
                     const int is = bf.refl[(f & 7) * g.Nvp + vt * VC + v];
-                    const T* p = bf.phi_in + (size_t)(is / VC) * (nn * N8) + (size_t)c * N8 + (is % VC);
+                    const T* p = phi + (size_t)(is / VC) * (nn * N8) + (size_t)c * N8 + (is % VC);
                     cp_async_elem(reinterpret_cast<T*>(&slot(SPH, r)) + v, p);
                     cp_async_elem(reinterpret_cast<T*>(&slot(SPH + 1, r)) + v, p + VC);
                 }
@@ -576,6 +587,11 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                 const int2 cl = cell(r);
                 if (cl.x < 0) continue;
                 const int fl = cl.y >> 16;
+                if (PRE && !(fl & 8)) {              // phibar+ as the pre-pass formed it
+                    Pg[cl.y & 0xffff] = slot(SPH, r);
+                    Pb[cl.y & 0xffff] = slot(SPH + 1, r);
+                    continue;
+                }
                 T cst[4 * NCV];
 #pragma unroll
                 for (int i = 0; i < NCV; ++i) {
@@ -626,7 +642,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                 }
                 if constexpr (TAB) pb = (hx + K::bc(cst[o + 1])) * ge;
                 K pg = ge;
-                if (!(fl & 8)) {
+                if (!PRE && !(fl & 8)) {
                     const K dg = slot(SPH, r) - ge, db = slot(SPH + 1, r) - pb;
                     pg = fma4(K::bc(cst[o + 2]), dg, ge);
                     pb = fma4(K::bc(cst[o + 3]), db, pb);
@@ -742,7 +758,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
 #pragma unroll 1
             for (int side = 0; side < 2; ++side)
                 if (side ? oa + tdim >= g.n[a] : oa == 0)
-                    edge_pass<T, D, TL, TAB, NOSRC, SK>(g, bf, org[0], org[1], org[2], a, side, j0, j1,
+                    edge_pass<T, D, TL, TAB, NOSRC, SK, PRE>(g, bf, org[0], org[1], org[2], a, side, j0, j1,
                                                         __ldg(bf.slots + (grp * 3 + a) * 2 + (side ? 0 : 1)),
                                                         reinterpret_cast<T*>(smem));
         }
@@ -752,15 +768,16 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
 // MIX = false: for instances without mixed visits, AL = false (TAB): whose
 // velocity rows are not whole chunks.  Each variant's loop holds only what it
 // needs: in 3D the registers and the loop's code size are the limit.
-template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true, bool AL = true>
+template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool MIX = true, bool AL = true,
+          bool PRE = false>
 __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (UOcc<T, D, T0_, T1_, T2_, TAB, SK>::value))
     k_usweep(const __grid_constant__ Geo g, const __grid_constant__ Bufs<T> bf) {
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_wait();
-    usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, MIX, AL>(g, bf, blockIdx.x, blockIdx.y, smem);
+    usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, MIX, AL, PRE>(g, bf, blockIdx.x, blockIdx.y, smem);
 }
 
-template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false>
+template <typename T, int D, int T0_, int T1_, int T2_, bool TAB, bool NOSRC, bool SK = false, bool PRE = false>
 __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (UOcc<T, D, T0_, T1_, T2_, TAB, SK>::value))
     k_usweep_batch(const Item* __restrict__ items, const Inst<T>* __restrict__ insts, const int* __restrict__ cur) {
     extern __shared__ __align__(128) unsigned char smem[];
@@ -772,7 +789,7 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (UOcc<T, D, T0_, T
     if (TAB && !rec.g.xal)
         usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, true, !TAB>(rec.g, rec.b, it.tile, it.grp, smem);
     else
-        usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK>(rec.g, rec.b, it.tile, it.grp, smem);
+        usweep_body<T, D, T0_, T1_, T2_, TAB, NOSRC, SK, true, true, PRE>(rec.g, rec.b, it.tile, it.grp, smem);
 }
 
 }  // namespace cdg
