@@ -150,20 +150,27 @@ void set_tiles(cdugks* h, int id) {
 int groups_for(const cdugks* h, int requested) {
     const Geo& g = h->g;
     if (requested > 0) return std::min(requested, g.NVT);
-    // The split of least cost, in chunks of one CTA's work: the chunks, times how
-    // far the last wave of CTAs (152 SMs, as many per SM as sweep A runs) is from
-    // full, plus what every group adds (its partial sums in the face and cell
-    // kernels, the CTAs' prologues: about 3.5 chunks in FP32, 0.5 of the slower FP64
-    // ones).
+    // The split of least cost, in chunks of one CTA's work: the chunks of a CTA
+    // (between the mean, which counts where the SM's pipes are busy, and the most,
+    // which counts where a CTA's own latency does), times the waves of CTAs (152 SMs,
+    // as many per SM as sweep A runs), plus what every group adds: its partial sums
+    // in the face and cell kernels and the CTAs' prologues, about 3.5 chunks in FP32
+    // and 0.5 of the slower FP64 ones; where few tiles leave the chip idle the face
+    // and cell kernels' serial sums over the groups count instead, in FP32 about a
+    // quarter of what a CTA needs for a chunk (FP64: not over the above).  A step
+    // with this split (groups): FP64, 64 x 64 cells x 24 x 24 velocities 0.79 ms (9),
+    // 0.90 (19); FP32 2D, 86 x 86 x 45 x 45 0.27 ms (9), 0.38 (64); FP32 1D, 8192 x
+    // 129 34 us (9), 61 (33); 400 x 128 27 us (11), 33 (32).
     const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2];
     const long long slots = 152LL * (h->prec == CDUGKS_FP32 ? cdg::sweep_a_ctas_f32(g.D, g.tile_id)
                                                             : cdg::sweep_a_ctas_f64(g.D, g.tile_id));
-    const double per_group = h->prec == CDUGKS_FP32 ? 3.5 : 0.5;
+    const double per_group = h->prec == CDUGKS_FP32 ? std::max(3.5, 0.23 * (double)slots / (double)tiles) : 0.5;
     long long G = 1;
     double best = 0.0;
     for (long long n = 1; n <= std::min(g.NVT, 64); ++n) {
         const long long ctas = tiles * n, waves = (ctas + slots - 1) / slots;
-        const double cost = (double)g.NVT * (double)(waves * slots) / (double)ctas + per_group * (double)n;
+        const double chunks = 0.5 * ((double)g.NVT / (double)n + (double)((g.NVT + n - 1) / n));
+        const double cost = chunks * (double)(waves * slots) / (double)tiles + per_group * (double)n;
         if (n == 1 || cost < best) {
             best = cost;
             G = n;
@@ -296,6 +303,9 @@ void set_groups(cdugks* h, int G) {
     const int mode = tile_mode(h->prec, g.D, g.tile_id);
     g.upw = cdg::mode_upwind(mode) && !((cdg::mode_sk(mode) || cdg::mode_acc(mode)) && h->zero_node);
     if (!g.upw) return;
+    // (these sweeps split visits and chunks evenly; the heat flux's raw moments go
+    // by ntpg chunks a group)
+    if (!cdg::mode_sk(mode)) g.G = G;
     h->slots.assign((size_t)g.G * 6, -1);
     for (int a = 0; a < 3; ++a) g.ws[a] = 0;
     for (int gr = 0; gr < g.G; ++gr)
@@ -1408,8 +1418,7 @@ int batch_plan(cdugks_batch* b) {
             std::stable_sort(v.begin(), v.end(), [&](const Item& x, const Item& y) {
                 const Geo& gx = b->mem[x.inst]->g;
                 const Geo& gy = b->mem[y.inst]->g;
-                const int wx = std::min(gx.ntpg, gx.NVT - x.grp * gx.ntpg), wy = std::min(gy.ntpg, gy.NVT - y.grp * gy.ntpg);
-                return wx > wy;
+                return (long long)gx.NVT * gy.G > (long long)gy.NVT * gx.G;      // chunks per item
             });
     // face and cell ranges: whole blocks of the kernel that runs them (64 threads,
     // or the persistent shape's threads), sized so that the batch has about 2048
