@@ -281,13 +281,14 @@ struct Shape {
         }
         if (!up) {      // (a shape with upwind owners: a node at 0, see OLD_A, and the wait hook)
             const TmaPair tma = make_tma<T, D, typename SM::TL>(g, SM::stage(false) ? phi_in : nullptr);
+            const dim3 og(grid.x, (unsigned)((g.NVT + g.ntpg - 1) / g.ntpg));      // its groups: ntpg chunks each
             if constexpr (NS && !UP) {
                 if (ns)
-                    e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>, grid, dim3(TL::NT), SM::bytes(false), s, in,
+                    e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE_NS>, og, dim3(TL::NT), SM::bytes(false), s, in,
                                    cur, tma);
             }
             if (!ns || UP)
-                e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE>, grid, dim3(TL::NT), SM::bytes(false), s, in, cur, tma);
+                e = launch_pdl(k_sweep<T, D, TX, TY, TZ, false, MODE>, og, dim3(TL::NT), SM::bytes(false), s, in, cur, tma);
         }
         if (e) return e;
         if (ev) cudaEventRecord(ev[1], s);
@@ -381,9 +382,9 @@ struct Shape {
     }
 };
 
-// A lean shape (lean.cuh): sweep A k_usweep, face constants (with the face
-// factor tables when XF), sweep B k_bflux (equilibria from them with XF), W update (with the
-// cell factor tables).  Single instances take the sweeps without the b-source
+// A lean shape: sweep A k_usweep with the cell factor tables, face constants (with
+// the face factor tables when XF), sweep B k_bflux (equilibria from them with XF), W
+// update (with the cell factor tables).  Single instances take the sweeps without the b-source
 // terms when the instance has none (Pr = 1); batched launches keep the general
 // ones.
 template <typename T, int D, int TX, int TY, int TZ, bool XF = true>

@@ -75,3 +75,23 @@ def test_acceleration_along_each_axis_matches_oracle(oracle_mod, nv, acc, prec):
         s.init(f)
         s.step(3)
         check(s, o, prec, groups)
+
+
+def test_wait_hook_with_groups_of_uneven_chunks(oracle_mod):
+    """The wait hook's staging sweep takes equal chunks a group (6 groups for the 7
+    that the sweeps with upwind owners take of 16 chunks); the handle recovers."""
+    cfg, f = wl.random_smooth(dim=2, n=(72, 28), nv=(8, 8), seed=1, amp=0.3, kn=3e-3)
+    s = cdugks.Solver(cfg, precision=cdugks.FP32, tile_id=cdugks.find_tile(cdugks.FP32, 2, (32, 8), 4), velocity_groups=7)
+    assert s.info().velocity_groups == 7
+    lib = cdugks.load()
+    s.init(f)
+    assert lib.cdugks_test_wait_timeout(s._h, 1) == 0
+    s.step(1)
+    assert s.sync_status() == cdugks.ERR_TIMEOUT
+    assert lib.cdugks_test_wait_timeout(s._h, 0) == 0
+    s.init(f)
+    s.step(3)
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(3)
+    check(s, o, cdugks.FP32, 7)
