@@ -5,16 +5,19 @@
 //   sweep A   per (tile of cells, group of velocity chunks): finalise phi^n from
 //             the stored pre-update value phi* (the last factor of eq. phiupdate,
 //             deferred until W^n is known), form phibar+ (eq. phibarplus) on the
-//             tile and its two-cell halo in shared memory, van Leer slopes
-//             (eq. VanLeer), reconstruct phibar at the owned faces along the
-//             characteristic (eq. relation) and sum the face conserved variables
-//             (eqs. rhobar-rhoEbar) over the group's velocities.
+//             tile and its halo in shared memory, van Leer slopes (eq. VanLeer),
+//             reconstruct phibar at the faces along the characteristic (eq.
+//             relation) and sum the face conserved variables (eqs.
+//             rhobar-rhoEbar) over the group's velocities.  The face-store
+//             shapes of the upwind-cell reconstruction run usweep.cuh's (a cell
+//             forms the faces it is upwind of), the others the one here (a tile
+//             forms its cells' left faces on a two-cell halo).
 //   face      sum the groups' partial face W; face constants (u, T, tau).
 //   sweep B   the face equilibrium (eqs. geq, beq), the inverse of eq. phibar,
 //             the microflux xi.n phi (eq. flux), its moments (for W) and the
 //             per-velocity net flux that gives phi* of eq. phiupdate, written to
 //             the other state buffer.  In the face-store modes sweep A keeps the
-//             reconstructed face values and sweep B is k_flux, which reads them;
+//             reconstructed face values and sweep B is bflux.cuh's, which reads them;
 //             otherwise sweep B reconstructs them again.
 //
 //   W update  W^{n+1} = W^n - dt sum_faces (M_right - M_left)/dx (eqs.
@@ -822,25 +825,25 @@ __device__ __forceinline__ void tma_load_4d(void* dst, const CUtensorMap* map, u
 // B) takes phibar+ and the slopes from: 0 forms both on the halo box itself;
 // 1 (prepared) loads phibar+ formed by k_prep and forms the slopes; 2 (stored)
 // loads phibar+ and the slopes formed by k_shslope.  Bit 2 (face store):
-// sweep A also writes the reconstructed face values, and sweep B is k_flux,
+// sweep A also writes the reconstructed face values, and sweep B is bflux.cuh's,
 // which reads them instead of reconstructing them again.
 // Bit 3 (face gradient): the paper's variant of the reconstruction, which also
 // carries the slopes to the face with their own limited derivatives (three
 // halo layers; fused face-store shapes only).
-// Bit 4 (Shakhov): the sweeps and k_flux evaluate the Shakhov equilibria
+// Bit 4 (Shakhov): the sweeps evaluate the Shakhov equilibria
 // (face-store shapes only); k_faceq and k_cellq add the raw moments the heat
 // flux needs.
 // Bit 5 (acceleration): k_prep adds the force terms of the sources (prepared
-// face-store shapes only) and k_flux takes them at the faces and in phi*.
+// face-store shapes only) and sweep B takes them at the faces and in phi*.
 // Bit 6 (launch-time, not a tile shape): the instance has no b-source, so
-// sweep A and k_flux leave out Z = xi.u - u^2/2 and its terms (whose
+// the sweeps leave out Z = xi.u - u^2/2 and its terms (whose
 // coefficients are then exactly 0: the same results, fewer instructions).
-// Bit 7 (lean): the face-store shapes whose sweep A is lean.cuh's (D = 2, 3; the
-// two-time model, upwind-cell reconstruction, velocity grids without a node at
-// xi_a = 0): its cell equilibria are products of per-axis Maxwellian factors
-// formed in double, kept in tables of every cell.  Bit 8 (face tables): sweep B
-// is lean.cuh's as well and takes the face equilibria from factor tables of
-// every face; without it sweep B is k_flux (an FP32 exponential per point).
+// Bit 7 (lean): the face-store shapes (D = 2, 3; the two-time model, upwind-cell
+// reconstruction, velocity grids without a node at xi_a = 0) whose sweep A takes
+// its cell equilibria as products of per-axis Maxwellian factors formed in
+// double, kept in tables of every cell.  Bit 8 (face tables): sweep B takes the
+// face equilibria from factor tables of every face as well; without it, an FP32
+// exponential per point.
 enum {
     MODE_FUSED = 0, MODE_PREP = 1, MODE_STORED = 2, MODE_FACES = 4, MODE_R2 = 8, MODE_SK = 16, MODE_ACC = 32,
     MODE_NOSRC = 64, MODE_LEAN = 128, MODE_XF = 256
@@ -1303,7 +1306,7 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT) k_shslope(const In
     }
 }
 
-// ---- pieces shared by the recomputing sweep B and k_flux
+// ---- pieces shared by the recomputing sweep B and bflux.cuh's
 
 // First owned cell of tile number `tile` (tiles numbered x fastest).
 template <typename TL, int D>
@@ -1510,7 +1513,7 @@ __device__ __forceinline__ void sweep_body(const Geo g, const Bufs<T> bf, int ti
     constexpr bool R2 = mode_r2(MODE);                           // face-gradient reconstruction
     constexpr bool SK = mode_sk(MODE);                           // Shakhov equilibria
     constexpr bool NOSRC = mode_nosrc(MODE);                     // no b-source (its terms left out)
-    static_assert(!(SWEEP_B && FACES), "sweep B of the face-store shapes is k_flux");
+    static_assert(!(SWEEP_B && FACES), "sweep B of the face-store shapes is k_bflux");
     static_assert(!SK || (FACES && !R2 && mode_source(MODE) != MODE_PREP), "Shakhov shapes are fused or stored face-store shapes");
     static_assert(!R2 || (FACES && !PREP), "the face-gradient reconstruction is built for fused face-store shapes");
     constexpr int PN = SM::PN;
@@ -2089,7 +2092,7 @@ __device__ __forceinline__ void sweep_body(const Geo g, const Bufs<T> bf, int ti
                     T sm[NM];
 #pragma unroll
                     for (int m = 0; m < NM; ++m) sm[m] = T(0);
-                    if (FACES) {   // sweep A computes each face once: keep it for k_flux
+                    if (FACES) {   // sweep A computes each face once: keep it for sweep B
                         int qf[3] = {qa[0], qa[1], qa[2]};
                         qf[a] += side;
                         T* const dst = bf.face[a] + face_addr(g, a, face_index(g, a, qf), vt);

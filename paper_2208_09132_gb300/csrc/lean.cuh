@@ -1,25 +1,15 @@
-// lean.cuh -- the "lean" face-store shapes of the CDUGKS step (arXiv:2208.09132,
-// Sec. 2.1) for D = 2 and 3.
+// lean.cuh -- equilibria from factor tables, for the "lean" face-store shapes of
+// the CDUGKS step (arXiv:2208.09132, Sec. 2.1; D = 2 and 3, velocity grids with
+// no node at xi_a = 0).
 //
-// They compute the same scheme as the fused face-store shapes (two relaxation
-// times, upwind-cell reconstruction; the velocity grid has no node at xi_a = 0)
-// with three differences in how:
-//
-//  * The equilibria (eqs. geq, beq) are products of separable factors: the
-//    Maxwellian of a place is rho (2 pi RT)^{-D/2} prod_b exp(-(xi_b - u_b)^2 / 2RT),
-//    and the per-axis factors of every cell and face are formed in double by the
-//    FP64 kernels (write_factors: W update, face constants, init) into tables.
-//    A point's g_eq is then D - 1 multiplications of table entries -- no
-//    exponential per point, and the exponent is exact to double rounding at any
-//    Mach number.
-//  * Sweep A forms phibar+ only on the cells that some face's reconstruction
-//    reads (the upwind cells U of the tile's faces and their axis neighbours),
-//    and each upwind cell reconstructs the values of the faces it is upwind of
-//    (one limited slope vector per cell, each face value formed once) into
-//    shared memory; the owners of the faces then sum the face moments.
-//  * Sweep B (k_lflux) reads the stored face values of both faces of its cell
-//    along every axis and takes their equilibria from the face factor tables;
-//    no barrier in its chunk loop (a shared face is formed by both cells).
+// The equilibria (eqs. geq, beq) are products of separable factors: the Maxwellian
+// of a place is rho (2 pi RT)^{-D/2} prod_b exp(-(xi_b - u_b)^2 / 2RT), and the
+// per-axis factors of every cell (and, with face tables, face) are formed in double
+// by the FP64 kernels (write_factors: W update, face constants, init) into tables.
+// A point's g_eq is then D - 1 multiplications of table entries -- no exponential
+// per point, and the exponent is exact to double rounding at any Mach number.
+// Sweep A of these shapes is usweep.cuh's with TAB, sweep B bflux.cuh's (with face
+// tables: XF).
 #pragma once
 
 #include "kernels.cuh"
