@@ -257,7 +257,11 @@ struct Shape {
         const int ax = !ACC ? -1 : (g.acc[0] != 0.0 ? 0 : (g.acc[1] != 0.0 ? 1 : 2));
         const int axes = (g.acc[0] != 0.0) + (g.acc[1] != 0.0) + (g.acc[2] != 0.0);
         const int len = ax == 0 ? g.nv1[0] / VC : (ax > 0 ? g.nv1[ax] : 1);
-        if (ACC && g.xal && axes == 1 && g.NVT / len < 65536) {    // a line of the forced axis's chunks per block row
+        // a line of the forced axis's chunks per block row, where that leaves a block for
+        // every SM (in 1D the line is all of velocity space: 4096 cells x 128 velocities,
+        // FP64, 32 blocks: pre-pass and sweep A 0.25 ms against 0.15 by chunks)
+        const long long lines = (g.Nc + kPrepCells - 1) / kPrepCells * (g.NVT / len);
+        if (ACC && g.xal && axes == 1 && g.NVT / len < 65536 && lines >= 152) {
             const dim3 lg((unsigned)((g.Nc + kPrepCells - 1) / kPrepCells), (unsigned)(g.NVT / len));
             if constexpr (ACC) e = launch_pdl(k_prep_line<T, D>, lg, dim3(kPrepCells), 0, s, g, hb, ax, len);
             if (e) return e;
