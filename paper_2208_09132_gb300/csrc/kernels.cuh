@@ -219,22 +219,11 @@ template <> struct Num<double> {
     static __device__ __forceinline__ double expo(double x) { return exp(x); }
     static __host__ __device__ __forceinline__ double cexp_scale() { return 1.0; }
     static __host__ __device__ __forceinline__ double irt_scale() { return -2.0; }
-    // The quotient p / s for p > 0 (then |s| is neither tiny nor 0): the reciprocal
-    // from the hardware's estimate by one cubic step of the Newton family (y + y(e +
-    // e^2), e = 1 - s y), the quotient corrected by its residual (Markstein): six
-    // FP64 operations and no range checks.  A product of the one-sided differences
-    // below the normal range counts as 0, as does NaN (compared on the high word, off
-    // the FP64 pipe, which bounds sweep A in FP64).  Sweep A at 256 x 256 cells x 32 x
-    // 32 velocities: 9.26 ms with this, 10.8 with the divide.
+    // (The divide is branched around where no lane needs it: in directions along which
+    // the flow does not vary it costs nothing.)
     static __device__ __forceinline__ double vanleer(double s1, double s2) {
-        const double p = s1 * s2, s = s1 + s2;
-        double y;
-        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
-        const double e = __fma_rn(-s, y, 1.0);
-        y = __fma_rn(y, __fma_rn(e, e, e), y);
-        double q = p * y;
-        q = __fma_rn(__fma_rn(-s, q, p), y, q);
-        return (unsigned)__double2hiint(p) - 0x00100000u <= 0x7fe00000u ? q : 0.0;
+        double p = s1 * s2;
+        return p > 0.0 ? p / (s1 + s2) : 0.0;
     }
 };
 

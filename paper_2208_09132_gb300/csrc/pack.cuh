@@ -197,6 +197,26 @@ __device__ __forceinline__ Pk<double> ldv4(const double* p) {
     return r;
 }
 
+// The van Leer limiter of the sweeps with upwind owners.  FP64: the quotient p / s
+// for p > 0 (then |s| is neither tiny nor 0) from the hardware's estimate of the
+// reciprocal by one cubic step of the Newton family (y + y(e + e^2), e = 1 - s y),
+// corrected by its residual (Markstein): six FP64 operations and no range checks or
+// branch.  A product of the one-sided differences below the normal range counts as
+// 0, as does NaN (compared on the high word, off the FP64 pipe, which bounds sweep A
+// in FP64).  Sweep A at 256 x 256 cells x 32 x 32 velocities: 9.26 ms with this, 10.8
+// with the divide.  (k_sweep and k_shslope keep the divide: with flows flat along an
+// axis they skip it, and the 3D 4 x 4 x 4 shape was 9 % slower with this.)
+__device__ __forceinline__ float vanleer1(float s1, float s2) { return Num<float>::vanleer(s1, s2); }
+__device__ __forceinline__ double vanleer1(double s1, double s2) {
+    const double p = s1 * s2, s = s1 + s2;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
+    const double e = __fma_rn(-s, y, 1.0);
+    y = __fma_rn(y, __fma_rn(e, e, e), y);
+    double q = p * y;
+    q = __fma_rn(__fma_rn(-s, q, p), y, q);
+    return (unsigned)__double2hiint(p) - 0x00100000u <= 0x7fe00000u ? q : 0.0;
+}
 // Half van Leer slope times dx of four velocities: s1 s2 / (s1 + s2) where the
 // one-sided differences share a sign, else 0 (eq. VanLeer).
 __device__ __forceinline__ Pk<float> vanleer4(const Pk<float>& s1, const Pk<float>& s2) {
@@ -216,7 +236,7 @@ __device__ __forceinline__ Pk<float> vanleer4(const Pk<float>& s1, const Pk<floa
 __device__ __forceinline__ Pk<double> vanleer4(const Pk<double>& s1, const Pk<double>& s2) {
     Pk<double> r;
 #pragma unroll
-    for (int i = 0; i < VC; ++i) r.v[i] = Num<double>::vanleer(s1.v[i], s2.v[i]);
+    for (int i = 0; i < VC; ++i) r.v[i] = vanleer1(s1.v[i], s2.v[i]);
     return r;
 }
 template <typename T>

@@ -236,7 +236,7 @@ __device__ __noinline__ void edge_pass(const Geo& g, const Bufs<T>& bf, int org0
                 for (int k = 0; k < 2; ++k)
 #pragma unroll
                     for (int v = 0; v < VC; ++v) {
-                        const T hs = Num<T>::vanleer(ctr[k][v] - lo[k][v], hi[k][v] - ctr[k][v]);
+                        const T hs = vanleer1(ctr[k][v] - lo[k][v], hi[k][v] - ctr[k][v]);
                         base[k][v] = fma(vr[(4 + e) * VC + v], hs, base[k][v]);
                         if (e == a) hsa[k][v] = hs;
                     }
