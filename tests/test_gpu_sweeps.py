@@ -95,3 +95,22 @@ def test_wait_hook_with_groups_of_uneven_chunks(oracle_mod):
     o.init(f)
     o.step(3)
     check(s, o, cdugks.FP32, 7)
+
+
+@pytest.mark.parametrize("prec", [cdugks.FP32, cdugks.FP64])
+@pytest.mark.parametrize("n,nv,acc", [((64, 41), (32, 8), (0.4, 0.0)), ((64, 41), (32, 8), (0.0, -0.3)),
+                                      ((64, 41), (32, 9), (0.0, 0.3)), ((13, 12, 9), (8, 8, 8), (0.0, 0.0, 0.4)),
+                                      ((13, 12, 9), (8, 8, 8), (0.0, 0.3, 0.0)), ((13, 12, 9), (8, 8, 8), (0.5, 0.0, 0.0))])
+def test_acceleration_prepass_along_lines_matches_oracle(oracle_mod, n, nv, acc, prec):
+    """Enough lines for the pre-pass along the forced axis (152 blocks of cells x lines)."""
+    D = len(n)
+    cfg, f = wl.random_smooth(dim=D, n=n, nv=nv, seed=3, amp=0.2, kn=3e-3, vmax=5.0)
+    cfg = _bc(cfg, [(P, P), (S, S), (P, P)][:D])
+    cfg["accel"] = list(acc) + [0.0] * (3 - D)
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(3)
+    s = cdugks.Solver(cfg, precision=prec, velocity_groups=4)
+    s.init(f)
+    s.step(3)
+    check(s, o, prec, acc)
