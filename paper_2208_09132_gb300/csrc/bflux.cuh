@@ -58,8 +58,6 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
     constexpr int NM = 2 + D, NT = TL::NT, NF = BS::NF, NX = BS::NX, N8 = 2 * VC, NFV = BS::NFV, NOV = BS::NOV;
     constexpr bool NC = !PERS, PF = sizeof(T) == 4;
     constexpr bool NOZ = SK || NOSRC;
-    constexpr bool GQ = gauss_ratio<T, D>();
-    constexpr int qi = SK ? 2 * D + 8 : D + 7;
     K* const FC = reinterpret_cast<K*>(smem);               // [NFV][NF] face constants
     K* const OC = FC + (size_t)NFV * NF;                    // [NOV][NT] constants of the own cell
     K* const LC = OC + (size_t)NOV * NT;                    // 1/dx_a, -dt (converted once: conversions use the FP64 pipe)
@@ -164,7 +162,6 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
             for (int b = 0; b < D; ++b) cst[D + 7 + b] = fs.sq[b];
             cst[2 * D + 7] = fs.e2;
         }
-        if constexpr (GQ && !XF) cst[qi] = gauss_q(fs.cexp, (T)g.dxi[0]);
 #pragma unroll
         for (int i = 0; i < NFV; ++i) {
             const T x[VC] = {cst[4 * i], cst[4 * i + 1], cst[4 * i + 2], cst[4 * i + 3]};
@@ -195,7 +192,6 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
             for (int b = 0; b < D; ++b) cst[D + 7 + b] = cs.sq[b];
             cst[2 * D + 7] = cs.e2;
         }
-        if constexpr (GQ) cst[qi] = gauss_q(cs.cexp, (T)g.dxi[0]);
 #pragma unroll
         for (int i = 0; i < NOV; ++i) {
             const T x[VC] = {cst[4 * i], cst[4 * i + 1], cst[4 * i + 2], cst[4 * i + 3]};
@@ -206,9 +202,8 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
 #pragma unroll
         for (int m = 0; m < NM; ++m) RS[m * NX + t].zero();
 
-    T hL = SK ? g.consts<T>().ceb : T(0), dxi = GQ ? (T)g.dxi[0] : T(0);
+    T hL = SK ? g.consts<T>().ceb : T(0);
     if (SK) keep(hL);
-    if (GQ) keep(dxi);
     if (t == 0) {
         const T x[VC] = {(T)g.idx[0], (T)g.idx[1], (T)g.idx[2], (T)-g.dt};
         *LC = K::of(x);
@@ -348,7 +343,7 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                 ge = table(bf.xf[a], g.nf[a], f, j);
                 be = (vr[3] + K::bc(cst[oe])) * ge;
             } else {
-                eq4<T, D, SK>(cst, vr, vr[3], hL, dxi, ge, be);
+                eq4<T, D, SK>(cst, vr, vr[3], hL, ge, be);
             }
             const K dg = pg - ge;
             K gf = fma4(K::bc(cst[oa]), dg, ge), gg, gb;
@@ -442,7 +437,7 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                 ge = table(bf.xc, g.Nc, cell, j);
                 be = (vr[3] + K::bc(cst[D + 2])) * ge;
             } else {
-                eq4<T, D, SK>(cst, vr, vr[3], hL, dxi, ge, be);
+                eq4<T, D, SK>(cst, vr, vr[3], hL, ge, be);
             }
             const K dg = gs - ge;
             const K ng = fma4(K::bc(lc[3]), dFg, fma4(K::bc(cst[D + 4]), dg, ge));

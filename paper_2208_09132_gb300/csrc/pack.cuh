@@ -248,61 +248,24 @@ __device__ __forceinline__ Pk<T> expo4(const Pk<T>& x) {
     return Pk<T>::of(v);
 }
 
-// FP64 in one dimension (the FP64 pipe is the bound, and the exponential most
-// of it): the four Maxwellian values of a chunk follow from the first two by
-// the recurrence of equally spaced nodes, E_{k+1} = E_k r_k, r_{k+1} = r_k q,
-// q = exp(2 cexp dxi^2) a constant of the place, kept as q - 1 (its rounding, the
-// same in every chunk, then counts |q - 1| times) -- two exponentials instead of
-// four and a handful of roundings -- unless the first one is near underflow.
-template <typename T, int D>
-__host__ __device__ constexpr bool gauss_ratio() {
-    return sizeof(T) == 8 && D == 1;
-}
-template <typename T>
-__device__ __forceinline__ T gauss_q(T cexp, T dxi) {
-    return (T)expm1((double)Ar<T>::mul(T(2) * cexp, Ar<T>::mul(dxi, dxi)));
-}
-__device__ __forceinline__ Pk<double> gauss_chunk(double cexp, double u, double q /* - 1 */, double dxi, const Pk<double>& xi) {
-    const double d0 = __dsub_rn(xi.v[0], u);
-    const double e0 = exp(__dmul_rn(cexp, __dmul_rn(d0, d0)));
-    Pk<double> r;
-    r.v[0] = e0;
-    if (e0 > 1e-280) {
-        double f = exp(__dmul_rn(cexp, __dmul_rn(dxi, __fma_rn(2.0, d0, dxi))));
-#pragma unroll
-        for (int i = 1; i < VC; ++i) {
-            r.v[i] = __dmul_rn(r.v[i - 1], f);
-            f = __fma_rn(f, q, f);
-        }
-    } else {
-#pragma unroll
-        for (int i = 1; i < VC; ++i) {
-            const double d = __dsub_rn(xi.v[i], u);
-            r.v[i] = exp(__dmul_rn(cexp, __dmul_rn(d, d)));
-        }
-    }
-    return r;
-}
-__device__ __forceinline__ Pk<float> gauss_chunk(float, float, float, float, const Pk<float>& xi) { return xi; }   // (unused)
-
 // The equilibria of a chunk's velocities xi (hx = |xi|^2 / 2) at a place with
 // the constants c: u (D), cexp, pref, eb, hu2, three more, with SK sq (D) and
-// e2, with gauss_ratio q - 1.  hL as in shakhov_point, dxi the axis-0 spacing.
+// e2.  hL as in shakhov_point.  One exponential per velocity: a chunk's four
+// values by the recurrence of equally spaced nodes from the first would take two
+// exponentials (FP64 1D, 8192 x 129: a step 0.325 ms instead of 0.372), but lose
+// what it climbs, exp(dxi^2 / RT): 1e-9 of the largest value at nodes four
+// thermal widths apart, all digits from six on.
 template <typename T, int D, bool SK>
-__device__ __forceinline__ void eq4(const T* c, const Pk<T>* xi, const Pk<T>& hx, T hL, T dxi, Pk<T>& ge, Pk<T>& be) {
+__device__ __forceinline__ void eq4(const T* c, const Pk<T>* xi, const Pk<T>& hx, T hL, Pk<T>& ge, Pk<T>& be) {
     using K = Pk<T>;
     K c2, cq;
-    if constexpr (!gauss_ratio<T, D>() || SK) {
 #pragma unroll
-        for (int a = 0; a < D; ++a) {
-            const K d = xi[a] - K::bc(c[a]);
-            c2 = a == 0 ? d * d : fma4(d, d, c2);
-            if constexpr (SK) cq = a == 0 ? K::bc(c[D + 7]) * d : fma4(K::bc(c[D + 7 + a]), d, cq);
-        }
+    for (int a = 0; a < D; ++a) {
+        const K d = xi[a] - K::bc(c[a]);
+        c2 = a == 0 ? d * d : fma4(d, d, c2);
+        if constexpr (SK) cq = a == 0 ? K::bc(c[D + 7]) * d : fma4(K::bc(c[D + 7 + a]), d, cq);
     }
-    K gM;
-    if constexpr (gauss_ratio<T, D>()) gM = K::bc(c[D + 1]) * gauss_chunk(c[D], c[0], c[SK ? 2 * D + 8 : D + 7], dxi, xi[0]);
-    else gM = K::bc(c[D + 1]) * expo4<T>(K::bc(c[D]) * c2);
+    const K gM = K::bc(c[D + 1]) * expo4<T>(K::bc(c[D]) * c2);
     if constexpr (SK) {              // as shakhov_point
         const K P1 = fma4(c2, K::bc(c[D] * Num<T>::irt_scale()), K::bc(T(-(D + 2))));
         const K in = fma4(hx, P1, fma4(K::bc(hL), c2, K::bc(-c[2 * D + 7])));
@@ -316,7 +279,7 @@ __device__ __forceinline__ void eq4(const T* c, const Pk<T>* xi, const Pk<T>& hx
 // How many values those constants are.
 template <typename T, int D, bool SK>
 struct EqPack {
-    static constexpr int N = D + 7 + (SK ? D + 1 : 0) + (gauss_ratio<T, D>() ? 1 : 0);
+    static constexpr int N = D + 7 + (SK ? D + 1 : 0);
     static constexpr int NV = (N + 3) / 4;
 };
 

@@ -507,7 +507,6 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
             for (int a = 0; a < D; ++a) cst[D + 7 + a] = (refl & (1 << a)) ? -cs.sq[a] : cs.sq[a];
             cst[2 * D + 7] = cs.e2;
         }
-        if constexpr (gauss_ratio<T, D>()) cst[SK ? 2 * D + 8 : D + 7] = gauss_q(cs.cexp, (T)g.dxi[0]);
 #pragma unroll
         for (int i = 0; i < NCV; ++i) {
             const T x[VC] = {cst[4 * i], cst[4 * i + 1], cst[4 * i + 2], cst[4 * i + 3]};
@@ -524,7 +523,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
         ends |= (valid && qa[a] == 0 ? 1 : 0) << (2 * a);
         ends |= (valid && qa[a] == g.n[a] - 1 ? 2 : 0) << (2 * a);
     }
-    const T hL = SK ? g.consts<T>().ceb : T(0), dxi = gauss_ratio<T, D>() ? (T)g.dxi[0] : T(0);
+    const T hL = SK ? g.consts<T>().ceb : T(0);
     auto fstr = [&](int a) { return a == 0 ? 1 : (a == 1 ? g.fn[1][0] : g.fn[2][0] * g.fn[2][1]); };
 
     Sums<T, D * NM> acc;
@@ -645,7 +644,7 @@ __device__ __forceinline__ void usweep_body(const Geo& g, const Bufs<T>& bf, int
                         ge = K::of(y);
                     }
                 } else {
-                    eq4<T, D, SK>(cst, xi, hx, hL, dxi, ge, pb);
+                    eq4<T, D, SK>(cst, xi, hx, hL, ge, pb);
                 }
                 if constexpr (TAB) pb = (hx + K::bc(cst[o + 1])) * ge;
                 K pg = ge;
