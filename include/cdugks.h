@@ -339,7 +339,9 @@ CDUGKS_API int cdugks_test_wait_timeout(cdugks_t *h, int on);
  * bound and initialised, of one precision and dim; each keeps its own
  * workspace.  The batch needs a small caller-owned workspace for its tables
  * and runs on its own stream; do not touch the members on other streams
- * between cdugks_batch_bind and cdugks_batch_sync.  Members may use different
+ * between cdugks_batch_bind and cdugks_batch_sync.  A member's own group or tile
+ * change leaves the batch as it was planned (at creation or the last change of its
+ * members or mode).  Members may use different
  * tile shapes (up to 8) and physics: every fused shape (two-time or Shakhov
  * collision model, either reconstruction) and the acceleration shapes batch;
  * the prepared and stored shapes without acceleration do not.  Results of a

@@ -1257,8 +1257,11 @@ struct cdugks_batch {
     std::vector<QItem> faceq_items, cellq_items;   // Shakhov members: raw moments
     std::vector<unsigned char> insts;          // host image of the Inst<T> table
     std::vector<int> cur;
+    // the members' group slots (Bufs::slots) as of the plan, like their geometry in
+    // insts: a member's own table follows its later group and tile changes
+    std::vector<int> slots, slot_at;           // one after another; each member's first
     size_t off_insts, off_cur, off_sweep[cdg::kMaxBatchLists], off_sweep_b[cdg::kMaxBatchLists], off_face, off_cell, total;
-    size_t off_prep, off_faceq, off_cellq;
+    size_t off_prep, off_faceq, off_cellq, off_slots;
     unsigned char* base;
     cudaStream_t stream;
     bool bound;
@@ -1287,6 +1290,26 @@ void fill_insts(cdugks_batch* b) {
         in[i].b[0] = bufs<T>(b->mem[i], 0);
         in[i].b[1] = bufs<T>(b->mem[i], 1);
     }
+}
+
+// The instance table, the slots that it points to and the parities to the workspace.
+template <typename T>
+cudaError_t upload_insts(cdugks_batch* b) {
+    Inst<T>* in = reinterpret_cast<Inst<T>*>(b->insts.data());
+    const int* slots = reinterpret_cast<const int*>(b->base + b->off_slots);
+    for (size_t i = 0; i < b->mem.size(); ++i) {
+        in[i].b[0].slots = in[i].b[1].slots = slots + b->slot_at[i];
+        b->cur[i] = b->mem[i]->cur;
+    }
+    cudaError_t e = cudaMemcpyAsync(b->base + b->off_insts, b->insts.data(), b->insts.size(), cudaMemcpyHostToDevice, b->stream);
+    if (!e && !b->slots.empty())
+        e = cudaMemcpyAsync(b->base + b->off_slots, b->slots.data(), sizeof(int) * b->slots.size(), cudaMemcpyHostToDevice,
+                            b->stream);
+    if (!e) e = cudaMemcpyAsync(b->base + b->off_cur, b->cur.data(), sizeof(int) * b->cur.size(), cudaMemcpyHostToDevice, b->stream);
+    return e;
+}
+cudaError_t upload_insts(cdugks_batch* b) {
+    return b->prec == CDUGKS_FP32 ? upload_insts<float>(b) : upload_insts<double>(b);
 }
 
 BatchPlan plan_of(const cdugks_batch* b) {
@@ -1475,6 +1498,12 @@ int batch_plan(cdugks_batch* b) {
     if (b->prec == CDUGKS_FP32) fill_insts<float>(b);
     else fill_insts<double>(b);
     b->cur.assign(n, 0);
+    b->slots.clear();
+    b->slot_at.clear();
+    for (const cdugks* m : b->mem) {
+        b->slot_at.push_back((int)b->slots.size());
+        if (m->g.upw) b->slots.insert(b->slots.end(), m->slots.begin(), m->slots.end());
+    }
     if (b->pers) {
         // one list per step: every member's sweep A items, then the face, sweep B and W items
         if (b->tile_ids.size() != 1) return fail(CDUGKS_ERR_INVALID, "a persistent batch needs one tile shape");
@@ -1518,12 +1547,14 @@ int batch_plan(cdugks_batch* b) {
         b->off_cur = take(sizeof(int) * (size_t)b->pcap_mem);
         b->off_phead = take(sizeof(PHead));
         b->off_pitems = take(sizeof(PItem) * (size_t)b->pcap_items);
+        b->off_slots = take(sizeof(int) * 3 * (size_t)b->pcap_items);   // six a group, which has an item of A and of B
         b->off_pstate = take(sizeof(PState));
         b->total = off;
         return CDUGKS_OK;
     }
     b->off_insts = take(b->insts.size());
     b->off_cur = take(sizeof(int) * n);
+    b->off_slots = take(sizeof(int) * b->slots.size());
     for (size_t k = 0; k < b->sweep_items.size(); ++k) {
         b->off_sweep[k] = take(sizeof(Item) * b->sweep_items[k].size());
         b->off_sweep_b[k] = take(sizeof(Item) * b->sweep_b_items[k].size());
@@ -1558,13 +1589,7 @@ cudaError_t batch_upload_persist(cdugks_batch* b) {
 // members in place (the binding and any captured graph stay valid).
 int batch_rewrite_in_place(cdugks_batch* b) {
     cudaError_t e;
-    for (size_t i = 0; i < b->mem.size(); ++i) b->cur[i] = b->mem[i]->cur;
-    if ((e = cudaMemcpyAsync(b->base + b->off_insts, b->insts.data(), b->insts.size(), cudaMemcpyHostToDevice,
-                             b->stream)) ||
-        (e = cudaMemcpyAsync(b->base + b->off_cur, b->cur.data(), sizeof(int) * b->cur.size(), cudaMemcpyHostToDevice,
-                             b->stream)) ||
-        (e = batch_upload_persist(b)))
-        return cuda_fail(e, "rewrite persistent plan");
+    if ((e = upload_insts(b)) || (e = batch_upload_persist(b))) return cuda_fail(e, "rewrite persistent plan");
     return CDUGKS_OK;
 }
 
@@ -1657,13 +1682,8 @@ int cdugks_batch_bind(cdugks_batch_t* b, void* device_ptr, size_t bytes, void* c
     batch_drop_graph(b);
     b->base = static_cast<unsigned char*>(device_ptr);
     b->stream = static_cast<cudaStream_t>(cuda_stream);
-    for (size_t i = 0; i < b->mem.size(); ++i) b->cur[i] = b->mem[i]->cur;
     cudaError_t e;
-    if ((e = cudaMemcpyAsync(b->base + b->off_insts, b->insts.data(), b->insts.size(), cudaMemcpyHostToDevice,
-                             b->stream)) ||
-        (e = cudaMemcpyAsync(b->base + b->off_cur, b->cur.data(), sizeof(int) * b->cur.size(),
-                             cudaMemcpyHostToDevice, b->stream)))
-        return cuda_fail(e, "upload batch tables");
+    if ((e = upload_insts(b))) return cuda_fail(e, "upload batch tables");
     for (size_t k = 0; k < b->sweep_items.size() && !b->pers; ++k)
         if ((e = cudaMemcpyAsync(b->base + b->off_sweep[k], b->sweep_items[k].data(),
                                  sizeof(Item) * b->sweep_items[k].size(), cudaMemcpyHostToDevice, b->stream)) ||

@@ -1,0 +1,55 @@
+"""Velocity groups and tile shapes changed on bound handles: a member of a batch
+that is changed between batch steps (the batch keeps the plan that it was made
+with), and handles that change after the binding."""
+import numpy as np
+import pytest
+
+from paper_2208_09132_gb300 import cdugks, workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("prec", [cdugks.FP32, cdugks.FP64])
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("D,n,nv", [(1, (70,), (64,)), (1, (33,), (65,)), (2, (40, 9), (8, 6))])
+def test_batch_keeps_its_plan_when_a_member_changes_groups_or_tile(prec, persistent, D, n, nv):
+    """Bit for bit the batch whose members were left alone; the member then
+    steps alone with its own groups."""
+    cells, mode = {1: (64,), 2: (32, 8) if prec == cdugks.FP32 else (16, 8)}[D], 4
+    if persistent and D == 2 and prec == cdugks.FP64:
+        pytest.skip("no persistent shape")
+    t = cdugks.find_tile(prec, D, cells, mode)
+    assert t
+    cfg, f = wl.random_smooth(dim=D, n=n, nv=nv, seed=5, amp=0.2, kn=3e-3, vmax=5.0)
+
+    def run(change):
+        out = []
+        for first, later in ((1, 4), (4, 1), (3, 2)):
+            s = [cdugks.Solver(cfg, precision=prec, tile_id=t, velocity_groups=first) for _ in range(2)]
+            for x in s:
+                x.init(f)
+            b = cdugks.Batch(s, persistent=persistent)
+            b.step(2)
+            assert b.sync() == 0
+            if change:
+                s[0].set_velocity_groups(later)
+                assert s[0].info().velocity_groups == later
+                b.step(2)
+                assert b.sync() == 0
+                assert cdugks.load().cdugks_set_tile(s[1]._h, 0) == 0     # the recomputing sweeps
+                b.step(2)
+            else:
+                b.step(4)
+            assert b.sync() == 0
+            out += [x.moments() for x in s] + [d for x in s for d in x.distributions()]
+            if change:
+                for x in s:
+                    x.step(1)
+                    assert x.sync_status() == 0
+                assert np.isfinite(s[0].moments()).all()
+                tol = 1e-5 if prec == cdugks.FP32 else 1e-12
+                assert np.abs(s[0].moments() - s[1].moments()).max() <= tol * np.abs(s[1].moments()).max()
+        return out
+
+    for a, b in zip(run(True), run(False)):
+        assert np.array_equal(a, b)
