@@ -179,6 +179,17 @@ int groups_for(const cdugks* h, int requested) {
     return (int)G;
 }
 
+// The velocity groups that a workspace has room for: what it starts with, and
+// where that is the automatic count also four waves of CTAs (152 SMs, two CTAs
+// each), for groups chosen after the binding.
+int group_room(const cdugks* h, int requested) {
+    const Geo& g = h->g;
+    const int G = groups_for(h, requested);
+    if (requested > 0) return G;
+    const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2], waves = (4 * 2 * 152 + tiles - 1) / tiles;
+    return std::max(G, (int)std::min<long long>({waves, g.NVT, 64}));
+}
+
 // The visits of sweep A with upwind owners (usweep.cuh), sorted by their sides
 // and mixed axes, then (velocity rows of whole chunks) with the axis-0 chunk
 // varying slowest and axis 1 fastest, so that a place's axis-0 factors stay the
@@ -643,8 +654,8 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     set_tiles(h, 0);
     h->vel32 = cast_vec<float>(h->vel);
     h->gsel = 0;
-    h->gcap = groups_for(h, 0);
-    set_groups(h, h->gcap);
+    h->gcap = group_room(h, 0);
+    set_groups(h, groups_for(h, 0));
     make_layout(h);
     h->stream = nullptr;
     h->cur = 0;
@@ -657,8 +668,8 @@ int cdugks_set_velocity_groups(cdugks_t* h, int groups) {
     const int G = groups_for(h, groups);
     if (h->bound && G > h->gcap)
         return fail(CDUGKS_ERR_INVALID, "more velocity groups than the bound workspace was laid out for");
-    if (!h->bound && G > h->gcap) {
-        h->gcap = G;
+    if (!h->bound && group_room(h, groups) > h->gcap) {
+        h->gcap = group_room(h, groups);
         make_layout(h);
     }
     drop_graphs(h);
@@ -713,8 +724,8 @@ int cdugks_set_tile(cdugks_t* h, int tile_id) {
     const int G = groups_for(h, h->gsel);
     if (h->bound && G > h->gcap) set_groups(h, h->gcap);
     else {
-        if (!h->bound && G > h->gcap) {
-            h->gcap = G;
+        if (!h->bound && group_room(h, h->gsel) > h->gcap) {
+            h->gcap = group_room(h, h->gsel);
             make_layout(h);
         }
         set_groups(h, G);

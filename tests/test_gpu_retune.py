@@ -53,3 +53,26 @@ def test_batch_keeps_its_plan_when_a_member_changes_groups_or_tile(prec, persist
 
     for a, b in zip(run(True), run(False)):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec,n,nv", [(cdugks.FP64, 64, 12), (cdugks.FP32, 86, 45), (cdugks.FP32, 40, 16)])
+def test_bound_handle_takes_four_waves_of_groups(prec, n, nv):
+    """A workspace laid out for the automatic group count also has room for the
+    groups that fill 152 SMs x 2 CTAs four times over."""
+    from paper_2208_09132_gb300 import tune
+    cfg, f = wl.kelvin_helmholtz(n=n, nv=nv)
+    for t in {0, tune.default_choice(cfg, prec)[0]}:
+        cells = cdugks.tile_shape(prec, 2, t)[0]
+        tiles = -(-n // cells[0]) * -(-n // cells[1])
+        most = min(-(-1216 // tiles), 64, -(-nv * nv // 4))
+        s = cdugks.Solver(cfg, precision=prec, tile_id=t)
+        s.init(f)
+        s.step(2)
+        auto = s.moments()
+        s.set_velocity_groups(most)
+        s.init(f)
+        s.step(2)
+        assert s.sync_status() == 0
+        assert s.info().velocity_groups == most
+        tol = 1e-5 if prec == cdugks.FP32 else 1e-12
+        assert np.abs(s.moments() - auto).max() <= tol * np.abs(auto).max()
