@@ -260,18 +260,31 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                 gb = fma4(c, ub - db, gb);
             }
         } else {
-            double fac[3] = {g.acc[0], g.acc[1], g.acc[2]};
-            if (nowall) fac[a] = 0.0;
+            // lane by lane: the record holds each lane's node along every axis
             T x[VC], y[VC];
+#pragma unroll
             for (int v = 0; v < VC; ++v) {
                 x[v] = y[v] = T(0);
+                if (ri[4 + v] < 0) continue;                                 // padding
                 const int i = vt * VC + v;
-                if (i < g.nv1[0] * g.nv1[1] * g.nv1[2])
-                    force_gradient<T, D>(g, fac, i, [&](int n, T& gv, T& bv) {
-                        const T* p = base + (unsigned)(n / VC) * nf8 + (n % VC);
-                        gv = p[0];
-                        bv = p[VC];
-                    }, x[v], y[v]);
+#pragma unroll
+                for (int b = 0; b < D; ++b) {
+                    if (g.acc[b] == 0.0 || (b == a && nowall)) continue;
+                    const int k = b == 0 ? ri[4 + v] : (b == 1 ? ri[8 + v] - g.xrow[1] : ri[12 + v] - g.xrow[2]);
+                    const int st = b == 0 ? 1 : (b == 1 ? g.nv1[0] : g.nv1[0] * g.nv1[1]);
+                    T ug = T(0), ub = T(0), dg = T(0), db = T(0);
+                    auto at = [&](int n) { return base + (unsigned)(n / VC) * nf8 + (n % VC); };
+                    if (k + 1 < g.nv1[b]) {
+                        ug = at(i + st)[0];
+                        ub = at(i + st)[VC];
+                    }
+                    if (k >= 1) {
+                        dg = at(i - st)[0];
+                        db = at(i - st)[VC];
+                    }
+                    x[v] = fma(-cacc[ACC ? b : 0], ug - dg, x[v]);
+                    y[v] = fma(-cacc[ACC ? b : 0], ub - db, y[v]);
+                }
             }
             gg = K::of(x);
             gb = K::of(y);
