@@ -50,7 +50,11 @@ struct BOcc {
     static constexpr int value = v < 1 ? 1 : (v > 8 ? 8 : v);
 };
 
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK, bool NOSRC, bool XF, bool ACC = false, bool PERS = false>
+// ROWS (ACC): the velocity rows are whole chunks.  The other rows' force gradients,
+// lane by lane, are in a kernel of their own: beside them the chunk-wide ones lack
+// registers (24^3 cells x 12^3 velocities, FP32: sweep B 0.64 -> 0.76 ms).
+template <typename T, int D, int T0_, int T1_, int T2_, bool SK, bool NOSRC, bool XF, bool ACC = false, bool PERS = false,
+          bool ROWS = true>
 __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int tile, int grp, unsigned char* smem) {
     using BS = BSmem<T, D, T0_, T1_, T2_, SK, XF>;
     using TL = typename BS::TL;
@@ -232,7 +236,7 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
         const unsigned long long nf8 = (unsigned long long)(unsigned)g.nf[a] * N8;
         const int vt = ri[0];
         gg = gb = K::bc(T(0));
-        if (g.xal) {
+        if constexpr (ROWS) {
             const int n0c = g.nv1[0] / VC;
 #pragma unroll
             for (int b = 0; b < D; ++b) {
@@ -258,6 +262,7 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                 const K c = K::bc(-cacc[ACC ? b : 0]);
                 gg = fma4(c, ug - dg, gg);
                 gb = fma4(c, ub - db, gb);
+                asm volatile("" ::: "memory");          // one axis's neighbours at a time: registers
             }
         } else {
             // lane by lane: the record holds each lane's node along every axis
@@ -477,12 +482,12 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
         for (int m = 0; m < NM; ++m) bf.mf[xa][((size_t)grp * NM + m) * (size_t)g.nf[xa] + xf] = RS[m * NX + t].value();
 }
 
-template <typename T, int D, int T0_, int T1_, int T2_, bool SK, bool NOSRC, bool XF, bool ACC = false>
+template <typename T, int D, int T0_, int T1_, int T2_, bool SK, bool NOSRC, bool XF, bool ACC = false, bool ROWS = true>
 __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (BOcc<T, D, T0_, T1_, T2_, SK, XF>::value))
     k_bflux(const __grid_constant__ Geo g, const __grid_constant__ Bufs<T> bf) {
     extern __shared__ __align__(128) unsigned char smem[];
     pdl_wait();
-    bflux_body<T, D, T0_, T1_, T2_, SK, NOSRC, XF, ACC>(g, bf, blockIdx.x, blockIdx.y, smem);
+    bflux_body<T, D, T0_, T1_, T2_, SK, NOSRC, XF, ACC, false, ROWS>(g, bf, blockIdx.x, blockIdx.y, smem);
 }
 
 template <typename T, int D, int T0_, int T1_, int T2_, bool SK, bool NOSRC, bool XF, bool ACC = false>
@@ -494,7 +499,10 @@ __global__ void __launch_bounds__(Tile<D, T0_, T1_, T2_>::NT, (BOcc<T, D, T0_, T
     pdl_wait();
     const Item it = items[blockIdx.x];
     rec.load(insts[it.inst], cur[it.inst] & 1);
-    bflux_body<T, D, T0_, T1_, T2_, SK, NOSRC, XF, ACC>(rec.g, rec.b, it.tile, it.grp, smem);
+    if (ACC && !rec.g.xal)
+        bflux_body<T, D, T0_, T1_, T2_, SK, NOSRC, XF, ACC, false, !ACC>(rec.g, rec.b, it.tile, it.grp, smem);
+    else
+        bflux_body<T, D, T0_, T1_, T2_, SK, NOSRC, XF, ACC>(rec.g, rec.b, it.tile, it.grp, smem);
 }
 
 // The pre-pass of an acceleration along one axis on velocity rows of whole

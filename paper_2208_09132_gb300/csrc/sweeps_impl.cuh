@@ -110,6 +110,10 @@ struct BLaunch {
         if constexpr (!SK) {
             if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, false, XF, ACC>);
         }
+        if constexpr (ACC) {
+            if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, false, XF, true, false>);
+            if (!e) e = size(k_bflux<T, D, BX, BY, BZ, false, true, XF, true, false>);
+        }
         if constexpr (BATCH) {
             if (!e) e = size(k_bflux_batch<T, D, BX, BY, BZ, SK, SK, XF, ACC>);
         }
@@ -123,6 +127,11 @@ struct BLaunch {
         unsigned tiles = 1;
         for (int a = 0; a < D; ++a) tiles *= (unsigned)((g.n[a] + TL::tdim(a) - 1) / TL::tdim(a));
         const dim3 grid(tiles, g.G);
+        if constexpr (ACC) {
+            if (!g.xal)
+                return g.nosrc ? launch_pdl(k_bflux<T, D, BX, BY, BZ, false, true, XF, true, false>, grid, dim3(TL::NT), BS::bytes, s, g, hb)
+                               : launch_pdl(k_bflux<T, D, BX, BY, BZ, false, false, XF, true, false>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
+        }
         if constexpr (!SK) {
             if (!g.nosrc)
                 return launch_pdl(k_bflux<T, D, BX, BY, BZ, false, false, XF, ACC>, grid, dim3(TL::NT), BS::bytes, s, g, hb);
