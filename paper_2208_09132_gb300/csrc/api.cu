@@ -147,8 +147,12 @@ void set_tiles(cdugks* h, int id) {
     for (int a = 0; a < 3; ++a) g.tiles[a] = a < g.D ? (g.n[a] + ts.t[a] - 1) / ts.t[a] : 1;
 }
 
-int groups_for(const cdugks* h, int requested) {
-    const Geo& g = h->g;
+// Four waves of CTAs over 152 SMs, two CTAs each.
+int four_waves(const Geo& g) {
+    const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2], n = (4 * 2 * 152 + tiles - 1) / tiles;
+    return (int)std::min<long long>({n, g.NVT, 64});
+}
+int groups_for(const Geo& g, int prec, int requested) {
     if (requested > 0) return std::min(requested, g.NVT);
     // The split of least cost, in chunks of one CTA's work: the chunks of a CTA
     // (between the mean, which counts where the SM's pipes are busy, and the most,
@@ -161,33 +165,45 @@ int groups_for(const cdugks* h, int requested) {
     // with this split (groups): FP64, 64 x 64 cells x 24 x 24 velocities 0.79 ms (9),
     // 0.90 (19); FP32 2D, 86 x 86 x 45 x 45 0.27 ms (9), 0.38 (64); FP32 1D, 8192 x
     // 129 34 us (9), 61 (33); 400 x 128 27 us (11), 33 (32).
+    // Without the face store sweep B reconstructs the faces again: more than half of
+    // the step, at fewer CTAs per SM, so both sweeps' waves count, 2 : 3 (24^3 cells x
+    // 12^3 velocities, stored 8 x 4 x 4 tiles, FP32: 1.73 ms at the 8 groups of this,
+    // 2.00 at the 4 that fill sweep A alone, 1.95 at 12).  In FP64 these
+    // sweeps keep four waves: no cost of this form is as good at every size (64^2 x
+    // 16^2, 8 x 8 tiles: 1.33 ms at 16 groups, 1.52 at the 8 of least cost); the
+    // face-gradient sweep A in FP64, the most costly chunks of all, takes no fewer
+    // (4096 x 128: 0.230 ms at 32 groups, 0.266 at 16).
+    const int mode = tile_mode(prec, g.D, g.tile_id);
+    const bool faces = cdg::mode_faces(mode), f32 = prec == CDUGKS_FP32;
+    if (!faces && !f32) return four_waves(g);
     const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2];
-    const long long slots = 152LL * (h->prec == CDUGKS_FP32 ? cdg::sweep_a_ctas_f32(g.D, g.tile_id)
-                                                            : cdg::sweep_a_ctas_f64(g.D, g.tile_id));
-    const double per_group = h->prec == CDUGKS_FP32 ? std::max(3.5, 0.23 * (double)slots / (double)tiles) : 0.5;
+    const long long slots_a = 152LL * (f32 ? cdg::sweep_a_ctas_f32(g.D, g.tile_id) : cdg::sweep_a_ctas_f64(g.D, g.tile_id));
+    const long long slots_b = faces ? 0 : 152LL * cdg::sweep_b_ctas_f32(g.D, g.tile_id);
+    const double per_group = f32 ? std::max(3.5, 0.23 * (double)slots_a / (double)tiles) : 0.5;
     long long G = 1;
     double best = 0.0;
     for (long long n = 1; n <= std::min(g.NVT, 64); ++n) {
-        const long long ctas = tiles * n, waves = (ctas + slots - 1) / slots;
-        const double chunks = 0.5 * ((double)g.NVT / (double)n + (double)((g.NVT + n - 1) / n));
-        const double cost = chunks * (double)(waves * slots) / (double)tiles + per_group * (double)n;
+        const long long ctas = tiles * n, most = (g.NVT + n - 1) / n;
+        if (!faces && (g.NVT + most - 1) / most != n) continue;         // (these sweeps' groups are equal runs)
+        const double chunks = 0.5 * ((double)g.NVT / (double)n + (double)most);
+        double filled = (double)((ctas + slots_a - 1) / slots_a * slots_a);
+        if (!faces) filled = 0.4 * filled + 0.6 * (double)((ctas + slots_b - 1) / slots_b * slots_b);
+        const double cost = chunks * filled / (double)tiles + per_group * (double)n;
         if (n == 1 || cost < best) {
             best = cost;
             G = n;
         }
     }
-    return (int)G;
+    return !f32 && cdg::mode_r2(mode) ? std::max((int)G, four_waves(g)) : (int)G;
 }
+int groups_for(const cdugks* h, int requested) { return groups_for(h->g, h->prec, requested); }
 
 // The velocity groups that a workspace has room for: what it starts with, and
-// where that is the automatic count also four waves of CTAs (152 SMs, two CTAs
-// each), for groups chosen after the binding.
+// where that is the automatic count also four waves, for groups chosen after the
+// binding.
 int group_room(const cdugks* h, int requested) {
-    const Geo& g = h->g;
     const int G = groups_for(h, requested);
-    if (requested > 0) return G;
-    const long long tiles = (long long)g.tiles[0] * g.tiles[1] * g.tiles[2], waves = (4 * 2 * 152 + tiles - 1) / tiles;
-    return std::max(G, (int)std::min<long long>({waves, g.NVT, 64}));
+    return requested > 0 ? G : std::max(G, four_waves(h->g));
 }
 
 // The visits of sweep A with upwind owners (usweep.cuh), sorted by their sides
@@ -1908,6 +1924,7 @@ int noalloc_run(cdugks* h, const void* phi_in, void* phi_out, double* W, cudaStr
         g.tile_id = 0;
         const cdg::TileShape ts = tile_of(h->prec, g.D, 0);
         for (int a = 0; a < 3; ++a) g.tiles[a] = a < g.D ? (g.n[a] + ts.t[a] - 1) / ts.t[a] : 1;
+        g.G = groups_for(g, h->prec, h->gsel);
     }
     const int NM = 2 + g.D;
     unsigned char* base = nullptr;

@@ -45,6 +45,8 @@ TileShape b_tile_shape_f32(int D, int id);      // of sweep B's batched items
 TileShape b_tile_shape_f64(int D, int id);
 int sweep_a_ctas_f32(int D, int id);              // CTAs of sweep A per SM
 int sweep_a_ctas_f64(int D, int id);
+int sweep_b_ctas_f32(int D, int id);              // of sweep B
+int sweep_b_ctas_f64(int D, int id);
 size_t sweep_smem_f32(int D, int id);
 size_t sweep_smem_f64(int D, int id);
 // Sweep mode of a shape (MODE_FUSED / MODE_PREP / MODE_STORED): prepared and

@@ -9,6 +9,7 @@ int tile_count_f64(int D) { return shapes_of<double>(D).count; }
 TileShape tile_shape_f64(int D, int id) { return shapes_of<double>(D).shape(id); }
 TileShape b_tile_shape_f64(int D, int id) { return shapes_of<double>(D).b_shape(id); }
 int sweep_a_ctas_f64(int D, int id) { return shapes_of<double>(D).a_ctas(id); }
+int sweep_b_ctas_f64(int D, int id) { return shapes_of<double>(D).b_ctas(id); }
 size_t sweep_smem_f64(int D, int id) { return shapes_of<double>(D).smem(id); }
 int tile_mode_f64(int D, int id) { return shapes_of<double>(D).mode(id); }
 

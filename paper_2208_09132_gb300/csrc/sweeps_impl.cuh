@@ -370,6 +370,10 @@ struct Shape {
         if constexpr (UP) return UOcc<T, D, TX, TY, TZ, false, SK>::value;
         else return Occ<T, D, TX, TY, TZ, false, MODE>::value;
     }
+    static int b_ctas() {
+        if constexpr (FACES) return BOcc<T, D, BT::X, BT::Y, BT::Z, SK, false>::value;
+        else return Occ<T, D, TX, TY, TZ, true, MODE>::value;
+    }
 
     static constexpr bool persistent = PB;
     static cudaError_t persist(const PHead* head, const PItem* items, const Inst<T>* insts, int* cur, PState* st,
@@ -473,6 +477,7 @@ struct LeanShape {
     static TileShape shape() { return {{TL::T0, TL::T1, TL::T2}}; }
     static TileShape b_shape() { return BL::shape(); }
     static int a_ctas() { return UOcc<T, D, TX, TY, TZ, true>::value; }
+    static int b_ctas() { return BOcc<T, D, BT::X, BT::Y, BT::Z, false, XF>::value; }
 
     static constexpr bool persistent = false;
     static cudaError_t persist(const PHead*, const PItem*, const Inst<T>*, int*, PState*, int, int, int, cudaStream_t) {
@@ -497,6 +502,7 @@ struct ShapeList<> {
     static TileShape shape(int) { return {{0, 0, 0}}; }
     static TileShape b_shape(int) { return {{0, 0, 0}}; }
     static int a_ctas(int) { return 1; }
+    static int b_ctas(int) { return 1; }
     static size_t smem(int) { return 0; }
     static int mode(int) { return 0; }
     static bool persistent(int) { return false; }
@@ -525,6 +531,7 @@ struct ShapeList<H, R...> {
     static TileShape shape(int id) { return id == 0 ? H::shape() : Rest::shape(id - 1); }
     static TileShape b_shape(int id) { return id == 0 ? H::b_shape() : Rest::b_shape(id - 1); }
     static int a_ctas(int id) { return id == 0 ? H::a_ctas() : Rest::a_ctas(id - 1); }
+    static int b_ctas(int id) { return id == 0 ? H::b_ctas() : Rest::b_ctas(id - 1); }
     static size_t smem(int id) { return id == 0 ? H::smem_bytes() : Rest::smem(id - 1); }
     static int mode(int id) { return id == 0 ? H::mode : Rest::mode(id - 1); }
     static bool persistent(int id) { return id == 0 ? H::persistent : Rest::persistent(id - 1); }
@@ -545,6 +552,7 @@ struct ShapeOps {
     TileShape (*shape)(int);
     TileShape (*b_shape)(int);      // the tile of sweep B's batched items
     int (*a_ctas)(int);             // CTAs of sweep A per SM
+    int (*b_ctas)(int);             // of sweep B
     size_t (*smem)(int);
     int (*mode)(int);
     bool (*persistent)(int);
@@ -554,7 +562,7 @@ struct ShapeOps {
 };
 template <typename T, typename L>
 ShapeOps<T> ops_of() {
-    return {L::count, &L::shape, &L::b_shape, &L::a_ctas, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
+    return {L::count, &L::shape, &L::b_shape, &L::a_ctas, &L::b_ctas, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
             &L::template sweep_batch<T>, &L::template persist<T>};
 }
 const ShapeOps<float>& shapes_f32_1();
