@@ -60,7 +60,9 @@ struct Layout {
 enum { BUF_PHIBAR = 1, BUF_SLOPES = 2, BUF_FACES = 4, BUF_FORCE = 8, BUF_XTAB = 16, BUF_VISITS = 32, BUF_CHUNKS = 64 };
 int buffers_of(int mode) {
     int b = 0;
-    if (cdg::mode_upwind(mode)) b |= BUF_VISITS;
+    // (visits with every face store that a shape with upwind owners can follow on,
+    // so that a bound handle may change between them)
+    if (cdg::mode_faces(mode) && !cdg::mode_r2(mode)) b |= BUF_VISITS;
     if (cdg::mode_faces(mode)) b |= BUF_CHUNKS;
     if (cdg::mode_lean(mode)) b |= BUF_XTAB;
     if (cdg::mode_acc(mode)) b |= BUF_FORCE;

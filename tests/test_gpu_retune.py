@@ -76,3 +76,23 @@ def test_bound_handle_takes_four_waves_of_groups(prec, n, nv):
         assert s.info().velocity_groups == most
         tol = 1e-5 if prec == cdugks.FP32 else 1e-12
         assert np.abs(s.moments() - auto).max() <= tol * np.abs(auto).max()
+
+
+@pytest.mark.parametrize("nv", [(8, 8), (10, 9)])
+def test_bound_handle_changes_between_the_face_store_shapes(oracle_mod, nv):
+    """From the stored face store to the fused one (which has sweep A by upwind
+    owners) and back, after the binding."""
+    cfg, f = wl.random_smooth(dim=2, n=(70, 19), nv=nv, seed=4, amp=0.2, kn=3e-3, vmax=5.0)
+    stored, fused = (cdugks.find_tile(cdugks.FP32, 2, (32, 8), m) for m in (6, 4))
+    assert stored and fused
+    s = cdugks.Solver(cfg, precision=cdugks.FP32, tile_id=stored)
+    o = oracle_mod.Oracle(cfg)
+    s.init(f)
+    o.init(f)
+    for t in (stored, fused, stored, fused):
+        assert cdugks.load().cdugks_set_tile(s._h, t) == 0
+        s.step(2)
+        o.step(2)
+        assert s.sync_status() == 0
+        ref = o.moments()
+        assert (np.abs(s.moments() - ref).max(axis=0) / np.abs(ref).max(axis=0)).max() <= 1e-5
