@@ -99,12 +99,7 @@ struct cdugks {
     std::vector<double> vel;  // [Nvp][8]: xi_0, xi_1, xi_2, w, |xi|^2/2, 0, 0, 0
     std::vector<float> vel32; // the same table rounded to float (FP32 storage)
     std::vector<int> refl;    // [8][Nvp]
-    std::vector<int> vint;    // visits of sweep A (Bufs::vint, Bufs::vrec)
-    std::vector<double> vrec;
-    std::vector<float> vrec32;
-    std::vector<int> cint;    // chunk records of sweep B (Bufs::cint, Bufs::crec)
-    std::vector<double> crec;
-    std::vector<float> crec32;
+    int nvis, vcls[64];       // visits of sweep A with upwind owners, and how many of each class
     std::vector<int> slots;   // [gcap][3][2] (Bufs::slots)
     // captured steps (cdugks_capture): one graph per parity of the state buffer it starts from
     cudaGraph_t graph[2] = {nullptr, nullptr};
@@ -208,79 +203,78 @@ int group_room(const cdugks* h, int requested) {
     return requested > 0 ? G : std::max(G, four_waves(h->g));
 }
 
-// The visits of sweep A with upwind owners (usweep.cuh), sorted by their sides
-// and mixed axes, then (velocity rows of whole chunks) with the axis-0 chunk
-// varying slowest and axis 1 fastest, so that a place's axis-0 factors stay the
-// same over long runs; and the chunks in that last order for sweep B.  Padding
-// and nodes at xi_a = 0 are stored as negative; such a node is summed half on
-// either side.
-void build_visits(cdugks* h) {
-    const Geo& g = h->g;
-    const int D = g.D, DM = cdg::mixed_axes(D), mask = ((1 << D) - 1) & ~((1 << DM) - 1);   // axes with visits of their own
-    std::vector<unsigned char> pos(g.Nvp, 0), zero(g.Nvp, 0);      // bits per axis: xi_a > 0; xi_a = 0
-    for (int i = 0; i < g.Nvp; ++i)
-        for (int a = 0; a < D; ++a) {
-            const double x = i < h->Nv ? h->vel[(size_t)i * 8 + a] : 0.0;
-            pos[i] |= (unsigned char)((x > 0.0 ? 1 : 0) << a);
-            zero[i] |= (unsigned char)((x == 0.0 ? 1 : 0) << a);
-        }
-    struct Visit {
-        int key, vt, flags, own;       // own: the signs of its axes in mask
-    };
-    const int n0c = g.nv1[0] / VC, m = g.nv1[1] * g.nv1[2];
-    auto order = [&](int vt) { return g.xal ? (vt % n0c) * m + vt / n0c : vt; };
-    // sweep B: the same, but with an acceleration along one axis that axis's nodes
-    // fastest, so that the chunks of neighbouring nodes, which the force gradients
-    // read, follow each other (cache hits)
-    const int fa = !g.accel ? -1 : (g.acc[0] != 0.0 ? 0 : (g.acc[1] != 0.0 ? 1 : 2));
-    auto b_order = [&](int vt) {
-        if (!g.xal || fa == 0) return vt;
-        if (fa != 2) return order(vt);
-        return (vt % n0c * g.nv1[1] + vt / n0c % g.nv1[1]) * g.nv1[2] + vt / (n0c * g.nv1[1]);
-    };
-    std::vector<Visit> vis, chunks;
-    vis.reserve(g.NVT + 16);
-    chunks.resize(g.NVT);
-    for (int vt = 0; vt < g.NVT; ++vt) {
-        const unsigned char* ps = &pos[(size_t)vt * VC];
-        const unsigned char* zs = &zero[(size_t)vt * VC];
-        chunks[b_order(vt)] = Visit{0, vt, 0, 0};
-        unsigned seen = 0;
-        for (int v = 0; v < VC; ++v) {
-            const int own = ps[v] & mask;
-            if ((seen >> own) & 1) continue;
-            seen |= 1u << own;
-            unsigned flags = 0;
-            for (int a = 0; a < D; ++a) {
-                unsigned plus = 0, minus = 0;
-                bool z = false;
-                for (int w = 0; w < VC; ++w) {
-                    if ((ps[w] & mask) != own) continue;
-                    ((ps[w] >> a) & 1 ? plus : minus) |= 1u << w;
-                    z = z || (((zs[w] >> a) & 1) && vt * VC + w < h->Nv);
-                }
-                const bool both = a < DM && ((plus && minus) || z);
-                if (both) flags |= 9u << a | plus << (8 + 4 * a) | minus << (20 + 4 * a);
-                else flags |= (plus ? 1u << a | plus << (8 + 4 * a) : minus << (8 + 4 * a));
-            }
-            vis.push_back(Visit{order(vt), vt, (int)flags, own});
-        }
+// The visits of sweep A with upwind owners (usweep.cuh) of one chunk, given to
+// put(flags, own): one per sign pattern `own` among its lanes of the axes that a
+// visit is not mixed along.  Padding and nodes at xi_a = 0 are stored as
+// negative; such a node is summed half on either side.
+struct Signs {
+    int plus, zero;            // bits per axis: xi_a > 0; xi_a = 0
+};
+Signs signs_of(const cdugks* h, int i) {
+    Signs s = {0, 0};
+    for (int a = 0; a < h->g.D; ++a) {
+        const double x = i < h->Nv ? h->vel[(size_t)i * 8 + a] : 0.0;
+        s.plus |= (x > 0.0 ? 1 : 0) << a;
+        s.zero |= (x == 0.0 ? 1 : 0) << a;
     }
-    std::stable_sort(vis.begin(), vis.end(), [](const Visit& x, const Visit& y) {
-        const int cx = cdg::visit_class(x.flags), cy = cdg::visit_class(y.flags);
-        return cx != cy ? cx < cy : x.key < y.key;
-    });
-    h->g.nvis = (int)vis.size();
-    h->g.mixed = std::any_of(vis.begin(), vis.end(), [](const Visit& v) { return (cdg::visit_class(v.flags) & 56) != 0; });
-    // the records' values go to the storage precision's table only
-    auto records = [&](const std::vector<Visit>& list, int ni, int nv, std::vector<int>& ints, auto& vals) {
-        using V = typename std::decay<decltype(vals[0])>::type;
-        ints.assign((size_t)ni * list.size(), 0);
-        vals.assign((size_t)nv * VC * list.size(), V(0));
-        for (size_t j = 0; j < list.size(); ++j) {
+    return s;
+}
+int own_axes(int D) { return ((1 << D) - 1) & ~((1 << cdg::mixed_axes(D)) - 1); }
+template <typename F>
+void chunk_visits(const cdugks* h, int vt, F&& put) {
+    const int D = h->g.D, DM = cdg::mixed_axes(D), mask = own_axes(D);
+    Signs s[VC];
+    for (int v = 0; v < VC; ++v) s[v] = signs_of(h, vt * VC + v);
+    unsigned seen = 0;
+    for (int v = 0; v < VC; ++v) {
+        const int own = s[v].plus & mask;
+        if ((seen >> own) & 1) continue;
+        seen |= 1u << own;
+        unsigned flags = 0;
+        for (int a = 0; a < D; ++a) {
+            unsigned plus = 0, minus = 0;
+            bool z = false;
+            for (int w = 0; w < VC; ++w) {
+                if ((s[w].plus & mask) != own) continue;
+                ((s[w].plus >> a) & 1 ? plus : minus) |= 1u << w;
+                z = z || (((s[w].zero >> a) & 1) && vt * VC + w < h->Nv);
+            }
+            const bool both = a < DM && ((plus && minus) || z);
+            if (both) flags |= 9u << a | plus << (8 + 4 * a) | minus << (20 + 4 * a);
+            else flags |= (plus ? 1u << a | plus << (8 + 4 * a) : minus << (8 + 4 * a));
+        }
+        put((int)flags, own);
+    }
+}
+void count_visits(cdugks* h) {
+    h->nvis = 0;
+    std::memset(h->vcls, 0, sizeof h->vcls);
+    for (int vt = 0; vt < h->g.NVT; ++vt)
+        chunk_visits(h, vt, [&](int flags, int) {
+            ++h->vcls[cdg::visit_class(flags)];
+            ++h->nvis;
+        });
+}
+
+// The records of a list of visits or chunks (get(j), j < n), formed a block at a
+// time and copied to the device; their values in the storage precision.
+struct Visit {
+    int key, vt, flags, own;       // own: the signs of the axes of own_axes()
+};
+template <typename V, typename G>
+cudaError_t upload_records(const cdugks* h, int n, int ni, int nv, size_t at_int, size_t at_val, G&& get) {
+    const Geo& g = h->g;
+    const int D = g.D, mask = own_axes(D), block = 4096;
+    std::vector<int> ints;
+    std::vector<V> vals;
+    for (int j0 = 0; j0 < n; j0 += block) {
+        const int m = std::min(block, n - j0);
+        ints.assign((size_t)ni * m, 0);
+        vals.assign((size_t)nv * VC * m, V(0));
+        for (int j = 0; j < m; ++j) {
             int* vi = &ints[(size_t)ni * j];
             V* vr = &vals[(size_t)nv * VC * j];
-            const Visit& vs = list[j];
+            const Visit vs = get(j0 + j);
             vi[0] = vs.vt;
             vi[1] = vs.flags;
             for (int v = 0; v < VC; ++v) {
@@ -291,10 +285,11 @@ void build_visits(cdugks* h) {
                     vr[(4 + a) * VC + v] = (V)-rec[5 + a];
                 }
                 vr[3 * VC + v] = (V)rec[4];
+                const Signs s = signs_of(h, i);
                 if (nv == cdg::kChunkVecs) vr[7 * VC + v] = (V)rec[3];
-                else if ((pos[i] & mask) == vs.own)
+                else if ((s.plus & mask) == vs.own)
                     for (int a = 0; a < D; ++a) {
-                        const bool z = (zero[i] >> a) & 1, plus = (pos[i] >> a) & 1;
+                        const bool z = (s.zero >> a) & 1, plus = (s.plus >> a) & 1;
                         const double w = z ? 0.5 * rec[3] : rec[3];
                         if (z) vi[16] |= 1 << (4 * a + v);
                         if (!cdg::visit_mixed(vs.flags, a)) vr[(7 + a) * VC + v] = (V)w;
@@ -311,14 +306,55 @@ void build_visits(cdugks* h) {
             vi[2] = vi[8];
             vi[3] = vi[12];
         }
-    };
-    if (h->prec == CDUGKS_FP32) {
-        records(vis, cdg::kVisitInts, cdg::kVisitVecs, h->vint, h->vrec32);
-        records(chunks, cdg::kChunkInts, cdg::kChunkVecs, h->cint, h->crec32);
-    } else {
-        records(vis, cdg::kVisitInts, cdg::kVisitVecs, h->vint, h->vrec);
-        records(chunks, cdg::kChunkInts, cdg::kChunkVecs, h->cint, h->crec);
+        // (from pageable memory: staged before the call returns)
+        cudaError_t e = cudaMemcpyAsync(h->base + at_int + sizeof(int) * ni * (size_t)j0, ints.data(), sizeof(int) * ints.size(),
+                                        cudaMemcpyHostToDevice, h->stream);
+        if (!e)
+            e = cudaMemcpyAsync(h->base + at_val + sizeof(V) * nv * VC * (size_t)j0, vals.data(), sizeof(V) * vals.size(),
+                                cudaMemcpyHostToDevice, h->stream);
+        if (e) return e;
     }
+    return cudaSuccess;
+}
+
+// Sweep A's visits, sorted by their sides and mixed axes, then (velocity rows of
+// whole chunks) with the axis-0 chunk varying slowest and axis 1 fastest, so that a
+// place's axis-0 factors stay the same over long runs.
+template <typename V>
+cudaError_t upload_visits(const cdugks* h) {
+    const Geo& g = h->g;
+    const int n0c = g.nv1[0] / VC, m = g.nv1[1] * g.nv1[2];
+    std::vector<Visit> vis;
+    vis.reserve(h->nvis);
+    for (int vt = 0; vt < g.NVT; ++vt)
+        chunk_visits(h, vt, [&](int flags, int own) {
+            vis.push_back(Visit{g.xal ? (vt % n0c) * m + vt / n0c : vt, vt, flags, own});
+        });
+    std::stable_sort(vis.begin(), vis.end(), [](const Visit& x, const Visit& y) {
+        const int cx = cdg::visit_class(x.flags), cy = cdg::visit_class(y.flags);
+        return cx != cy ? cx < cy : x.key < y.key;
+    });
+    return upload_records<V>(h, (int)vis.size(), cdg::kVisitInts, cdg::kVisitVecs, h->lay.vint, h->lay.vrec,
+                             [&](int j) { return vis[j]; });
+}
+// Sweep B's chunks, in the same order without the classes, but with an
+// acceleration along one axis that axis's nodes fastest, so that the chunks of
+// neighbouring nodes, which the force gradients read, follow each other.
+template <typename V>
+cudaError_t upload_chunks(const cdugks* h) {
+    const Geo& g = h->g;
+    const int n0c = g.nv1[0] / VC, m = g.nv1[1] * g.nv1[2];
+    const int fa = !g.accel ? -1 : (g.acc[0] != 0.0 ? 0 : (g.acc[1] != 0.0 ? 1 : 2));
+    return upload_records<V>(h, g.NVT, cdg::kChunkInts, cdg::kChunkVecs, h->lay.cint, h->lay.crec, [&](int j) {
+        int vt = j;
+        if (g.xal && fa == 2) {                   // j = (c0 nv1_1 + k1) nv1_2 + k2
+            const int k2 = j % g.nv1[2], k1 = j / g.nv1[2] % g.nv1[1], c0 = j / m;
+            vt = c0 + n0c * (k1 + g.nv1[1] * k2);
+        } else if (g.xal && fa != 0) {            // j = c0 nv1_1 nv1_2 + k1 + nv1_1 k2
+            vt = j / m + n0c * (j % m);
+        }
+        return Visit{0, vt, 0, 0};
+    });
 }
 
 // The velocity groups, and the slots of the face-W partial sums: one per group
@@ -335,17 +371,27 @@ void set_groups(cdugks* h, int G) {
     // (these sweeps split visits and chunks evenly; the heat flux's raw moments go
     // by ntpg chunks a group)
     if (!cdg::mode_sk(mode)) g.G = G;
+    g.nvis = h->nvis;
+    g.mixed = 0;
+    for (int c = 0; c < 64; ++c) g.mixed = g.mixed || (h->vcls[c] && (c & 56));
     h->slots.assign((size_t)g.G * 6, -1);
     for (int a = 0; a < 3; ++a) g.ws[a] = 0;
-    for (int gr = 0; gr < g.G; ++gr)
+    for (int gr = 0; gr < g.G; ++gr) {
+        const long long j0 = (long long)gr * g.nvis / g.G, j1 = (long long)(gr + 1) * g.nvis / g.G;
+        bool has[3][2] = {{false, false}, {false, false}, {false, false}};
+        long long first = 0;                       // of the class
+        for (int c = 0; c < 64; ++c) {
+            if (first < j1 && first + h->vcls[c] > j0)
+                for (int a = 0; a < g.D; ++a) {
+                    has[a][cdg::visit_plus(c, a)] = true;
+                    if (cdg::visit_mixed(c, a)) has[a][0] = true;
+                }
+            first += h->vcls[c];
+        }
         for (int a = 0; a < g.D; ++a)
-            for (int side = 0; side < 2; ++side) {
-                bool has = false;
-                for (long long j = (long long)gr * g.nvis / g.G; j < (long long)(gr + 1) * g.nvis / g.G && !has; ++j)
-                    has = cdg::visit_plus(h->vint[cdg::kVisitInts * (size_t)j + 1], a) == side ||
-                          (!side && cdg::visit_mixed(h->vint[cdg::kVisitInts * (size_t)j + 1], a));
-                if (has) h->slots[(size_t)(gr * 3 + a) * 2 + side] = g.ws[a]++;
-            }
+            for (int side = 0; side < 2; ++side)
+                if (has[a][side]) h->slots[(size_t)(gr * 3 + a) * 2 + side] = g.ws[a]++;
+    }
 }
 
 void make_layout(cdugks* h) {
@@ -378,12 +424,12 @@ void make_layout(cdugks* h) {
     L.vel = take(h->elt * 8 * g.Nvp);
     L.refl = take(sizeof(int) * 8 * g.Nvp);
     const bool vis = (h->bufs_cap & BUF_VISITS) != 0;
-    L.vint = vis ? take(sizeof(int) * h->vint.size()) : 0;
-    L.vrec = vis ? take(h->elt * std::max(h->vrec.size(), h->vrec32.size())) : 0;
+    L.vint = vis ? take(sizeof(int) * cdg::kVisitInts * (size_t)h->nvis) : 0;
+    L.vrec = vis ? take(h->elt * cdg::kVisitVecs * VC * (size_t)h->nvis) : 0;
     L.slots = vis ? take(sizeof(int) * 6 * (size_t)h->gcap) : 0;
     const bool chk = (h->bufs_cap & BUF_CHUNKS) != 0;
-    L.cint = chk ? take(sizeof(int) * h->cint.size()) : 0;
-    L.crec = chk ? take(h->elt * std::max(h->crec.size(), h->crec32.size())) : 0;
+    L.cint = chk ? take(sizeof(int) * cdg::kChunkInts * (size_t)g.NVT) : 0;
+    L.crec = chk ? take(h->elt * cdg::kChunkVecs * VC * (size_t)g.NVT) : 0;
     L.io = take(sizeof(double) * std::max(NM, g.D * g.D + g.D) * g.Nc);   // moments, or P and q
     const bool sk = h->collision == CDUGKS_COLLISION_SHAKHOV;
     const int NQ = g.D + g.D * (g.D + 1) / 2;
@@ -668,7 +714,6 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     g.mirror = 1;
     for (int a = 0; a < D; ++a)
         for (int s = 0; s < 2; ++s) g.mirror = g.mirror && g.bc[a][s] != CDUGKS_BC_DIRICHLET;
-    build_visits(h);
     set_tiles(h, 0);
     h->vel32 = cast_vec<float>(h->vel);
     h->gsel = 0;
@@ -735,6 +780,7 @@ int cdugks_set_tile(cdugks_t* h, int tile_id) {
     if (need & ~h->bufs_cap) {
         if (h->bound)
             return fail(CDUGKS_ERR_INVALID, "this shape needs more workspace buffers: select it before cdugks_bind");
+        if (need & ~h->bufs_cap & BUF_VISITS) count_visits(h);
         h->bufs_cap |= need;
         make_layout(h);
     }
@@ -836,7 +882,6 @@ int cdugks_set_acceleration(cdugks_t* h, const double* a) {
     const Geo old = h->g;
     for (int b = 0; b < 3; ++b) h->g.acc[b] = acc[b];
     h->g.accel = on;
-    build_visits(h);             // (sweep B's chunk order)
     const int rc = cdugks_set_tile(h, id);
     if (rc) h->g = old;
     return rc;
@@ -878,23 +923,14 @@ int cdugks_bind(cdugks_t* h, void* device_ptr, size_t bytes, void* cuda_stream) 
     if ((e = cudaMemcpyAsync(h->base + h->lay.refl, h->refl.data(), h->refl.size() * sizeof(int),
                              cudaMemcpyHostToDevice, h->stream)))
         return cuda_fail(e, "upload reflection table");
-    if (h->bufs_cap & BUF_VISITS) {
-        const void* vr = h->prec == CDUGKS_FP32 ? static_cast<const void*>(h->vrec32.data())
-                                                : static_cast<const void*>(h->vrec.data());
-        if ((e = cudaMemcpyAsync(h->base + h->lay.vint, h->vint.data(), sizeof(int) * h->vint.size(),
-                                 cudaMemcpyHostToDevice, h->stream)) ||
-            (e = cudaMemcpyAsync(h->base + h->lay.vrec, vr, h->elt * std::max(h->vrec.size(), h->vrec32.size()),
-                                 cudaMemcpyHostToDevice, h->stream)))
+    const bool f32 = h->prec == CDUGKS_FP32;
+    try {
+        if ((h->bufs_cap & BUF_VISITS) && (e = f32 ? upload_visits<float>(h) : upload_visits<double>(h)))
             return cuda_fail(e, "upload visits");
-    }
-    if (h->bufs_cap & BUF_CHUNKS) {
-        const void* cr = h->prec == CDUGKS_FP32 ? static_cast<const void*>(h->crec32.data())
-                                                : static_cast<const void*>(h->crec.data());
-        if ((e = cudaMemcpyAsync(h->base + h->lay.cint, h->cint.data(), sizeof(int) * h->cint.size(),
-                                 cudaMemcpyHostToDevice, h->stream)) ||
-            (e = cudaMemcpyAsync(h->base + h->lay.crec, cr, h->elt * std::max(h->crec.size(), h->crec32.size()),
-                                 cudaMemcpyHostToDevice, h->stream)))
+        if ((h->bufs_cap & BUF_CHUNKS) && (e = f32 ? upload_chunks<float>(h) : upload_chunks<double>(h)))
             return cuda_fail(e, "upload chunk records");
+    } catch (const std::bad_alloc&) {
+        return fail(CDUGKS_ERR_OOM, "host allocation failed");
     }
     if ((e = cudaMemsetAsync(h->base + h->lay.status, 0, 256, h->stream))) return cuda_fail(e, "clear status");
     if ((e = cudaStreamSynchronize(h->stream))) return cuda_fail(e, "cudaStreamSynchronize");
