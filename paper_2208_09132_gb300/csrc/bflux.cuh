@@ -9,7 +9,9 @@
 // but twice the equilibria and inversions; the exchange costs one barrier per
 // chunk and 16 bytes in and 32 out of shared memory per face and field.)
 // The next chunk's phi* and face values are loaded to registers before the
-// barrier (FP32); two CTAs per SM keep enough of them in flight.
+// barrier (FP32); two CTAs per SM keep enough of them in flight.  Under an
+// acceleration the cell's own phi* and force come after the barrier: held over
+// the faces' gradients they cost spills (256^2 cells x 32^2 velocities 0.96 -> 0.86 ms).
 //
 // A face's moments are summed by the thread that forms it as a left face; a
 // face at the domain's high end by the thread beyond it, or (a tile that ends
@@ -128,13 +130,10 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
         }
         cp_async_commit();
     };
-    K fg[D], fb[D], og, ob, xg, xb, fog, fob;
+    K fg[D], fb[D], og, ob, xg, xb;
     auto load = [&](int vt) {
         const unsigned long long v = (unsigned)vt;
-        if (valid) {
-            load_gb<NC>(bf.phi_in + (v * (unsigned)g.Nc + (unsigned)cell) * N8, og, ob);
-            if constexpr (ACC) load_gb<NC>(bf.force + (v * (unsigned)g.Nc + (unsigned)cell) * N8, fog, fob);
-        }
+        if (!ACC && valid) load_gb<NC>(bf.phi_in + (v * (unsigned)g.Nc + (unsigned)cell) * N8, og, ob);
 #pragma unroll
         for (int a = 0; a < D; ++a)
             if ((mine >> a) & 1) load_gb<NC>(bf.face[a] + (v * (unsigned)g.nf[a] + (unsigned)ff[a]) * N8, fg[a], fb[a]);
@@ -420,12 +419,15 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                     RS[m * NX + t] = k;
                 }
         }
-        const K gs = og, bs = ob, fgs = fog, fbs = fob;
+        K gs, bs;
+        if constexpr (!ACC) gs = og, bs = ob;
         if (PF && j + 1 < j1) load(rec_int(j + 1)[0]);      // in flight over the rest of this chunk
         fetch_rec(j + 3);
         __syncthreads();
         if (TL::T0 >= 32 && lead && j + 2 < j1) hint(rec_int(j + 2)[0]);
         if (valid) {
+            const unsigned long long own = ((unsigned long long)(unsigned)vt * (unsigned)g.Nc + (unsigned)cell) * N8;
+            if constexpr (ACC) load_gb<NC>(bf.phi_in + own, gs, bs);
             K dFg, dFb;
             T lc[VC];
             LC->get(lc);
@@ -439,6 +441,8 @@ __device__ __forceinline__ void bflux_body(const Geo& g, const Bufs<T>& bf, int 
                 dFb = a == 0 ? ix * eb : fma4(ix, eb, dFb);
             }
             if constexpr (ACC) {     // + dt F^n (eq. phiupdate's source, rectangle rule)
+                K fgs, fbs;
+                load_gb<NC>(bf.force + own, fgs, fbs);
                 dFg = dFg - fgs;
                 dFb = dFb - fbs;
             }
