@@ -20,8 +20,8 @@
 // What bounds it: FP32 the 16 + 8 D B per point at 16 warps per SM; FP64 the FP64
 // pipe.  Against forming a face in both its cells, ms per launch: FP32 3D 48^3 cells
 // x 24^3 velocities 20.3 -> 13.7 (4.5 TB/s of its 40 B per point), 2D 256^2 x 32^2
-// 0.432 -> 0.392 (5.5 TB/s of 32 B), under an acceleration 1.70 -> 0.93; FP64 2D
-// 256^2 x 32^2 8.70 -> 6.64, 1D 8192 x 129 0.246 -> 0.143.
+// 0.432 -> 0.392 (5.5 TB/s of 32 B), under an acceleration 1.70 -> 0.86; FP64 2D
+// 256^2 x 32^2 8.70 -> 6.59, 1D 8192 x 129 0.246 -> 0.173.
 #pragma once
 
 #include "usweep.cuh"

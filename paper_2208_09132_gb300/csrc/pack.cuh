@@ -198,24 +198,38 @@ __device__ __forceinline__ Pk<double> ldv4(const double* p) {
 }
 
 // The van Leer limiter of the sweeps with upwind owners.  FP64: the quotient p / s
-// for p > 0 (then |s| is neither tiny nor 0) from the hardware's estimate of the
-// reciprocal by one cubic step of the Newton family (y + y(e + e^2), e = 1 - s y),
-// corrected by its residual (Markstein): six FP64 operations and no range checks or
-// branch.  A product of the one-sided differences below the normal range counts as
-// 0, as does NaN (compared on the high word, off the FP64 pipe, which bounds sweep A
-// in FP64).  Sweep A at 256 x 256 cells x 32 x 32 velocities: 9.26 ms with this, 10.8
-// with the divide.  (k_sweep and k_shslope keep the divide: with flows flat along an
-// axis they skip it, and the 3D 4 x 4 x 4 shape was 9 % slower with this.)
+// for p > 0 by residual correction with one FMA (P. Markstein, IBM J. Res. Dev. 34
+// (1990) 111): with an approximate reciprocal y of s and q = p y, twice
+// q <- q + (p - s q) y.  y is the FP32 reciprocal of the leading 24 bits of s (an
+// error of at most 2^-23 for the rest of s, 2^-23 for the 1 ulp of the instruction)
+// with the exponent of s put back, so a correction takes a relative error e to
+// 2^-22 e: 2^-22, 2^-44, 2^-66, each but the last beside its rounding of 2^-53.  The
+// result is the rounding of a value within 2^-65 of the quotient, off by at most
+// (1/2 + 2^-12) ulp: the correctly rounded quotient, or its neighbour where the
+// quotient lies within 2^-12 ulp of the middle between the two.  That takes products
+// whose residuals do not underflow and an s whose reciprocal is normal; all others
+// are divided.  Five operations of the FP64 pipe, which bounds sweep A in FP64, instead of
+// the divide's, and none where no lane's differences share a sign (flat flows):
+// sweep A at 256 x 256 cells x 32 x 32 velocities 8.67 ms, with the divide 10.64; 1D 8192 x
+// 129 0.152 with either.  (k_sweep and k_shslope keep the divide.)
 __device__ __forceinline__ float vanleer1(float s1, float s2) { return Num<float>::vanleer(s1, s2); }
+static __device__ __noinline__ double vanleer_divide(double p, double s) { return p / s; }
 __device__ __forceinline__ double vanleer1(double s1, double s2) {
     const double p = s1 * s2, s = s1 + s2;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(s));
-    const double e = __fma_rn(-s, y, 1.0);
-    y = __fma_rn(y, __fma_rn(e, e, e), y);
-    double q = p * y;
-    q = __fma_rn(__fma_rn(-s, q, p), y, q);
-    return (unsigned)__double2hiint(p) - 0x00100000u <= 0x7fe00000u ? q : 0.0;
+    const unsigned hp = (unsigned)__double2hiint(p), hs = (unsigned)__double2hiint(s), ls = (unsigned)__double2loint(s);
+    const unsigned es = hs & 0x7ff00000u;
+    double q = 0.0;
+    if (hp - 0x01700000u < 0x7e800000u && es < 0x7fc00000u) {       // 2^-1000 <= p < infinity, |s| < 2^1021
+        const unsigned r = __float_as_uint(Num<float>::rcp(__uint_as_float(0x3f800000u | (hs & 0xfffffu) << 3 | ls >> 29)));
+        // its exponent from FP32's bias to FP64's, less that of s
+        const double y = __hiloint2double((int)(((r >> 3) + 0x77f00000u - es) | (hs & 0x80000000u)), (int)(r << 29));
+        q = p * y;
+        q = __fma_rn(__fma_rn(-s, q, p), y, q);
+        q = __fma_rn(__fma_rn(-s, q, p), y, q);
+    } else if (hp < 0x7ff00001u && (hp | (unsigned)__double2loint(p)) != 0u) {   // positive all the same
+        q = vanleer_divide(p, s);
+    }
+    return q;
 }
 // Half van Leer slope times dx of four velocities: s1 s2 / (s1 + s2) where the
 // one-sided differences share a sign, else 0 (eq. VanLeer).

@@ -39,7 +39,7 @@
 // owners, ms per launch: FP32 3D 48^3 cells x 24^3 velocities 39.8 -> 14.2 (3.4 TB/s
 // of its 32 B per point), 45 x 37 x 29 x 14^3 between walls 7.3 -> 2.9, 2D 256^2 x
 // 32^2 0.615 -> 0.402 (4.0 TB/s), 100^2 x 101^2 with nodes at 0 1.71 -> 0.81; FP64
-// 2D 256^2 x 32^2 13.0 -> 9.3; 1D 8192 x 129 0.137 -> 0.134.
+// 2D 256^2 x 32^2 13.0 -> 8.7 (1D 8192 x 129 0.137 -> 0.152, at 7 groups instead of 17).
 #pragma once
 
 #include "kernels.cuh"
