@@ -76,9 +76,9 @@ def default_choice(cfg, precision):
             lean = 1 if mode & 256 else 2
         else:
             lean = -1
-        if D == 2 and precision == cdugks.FP32 and cells > 256:
-            cells = 0                  # one CTA of 512 threads per SM idles at every barrier: two of 256 measured faster
-        pref = (lean, mode & 3 == 0, cells if cells <= wl.ncells(cfg) else -cells)
+        # (2D FP32: one CTA of 512 threads per SM idles at every barrier, two of 256 are faster at every size)
+        fits = cells <= wl.ncells(cfg) and not (D == 2 and precision == cdugks.FP32 and cells > 256)
+        pref = (lean, mode & 3 == 0, cells if fits else -cells)
         if best is None or pref > best[0]:
             best = (pref, t)
     return (best[1] if best else 0), 0

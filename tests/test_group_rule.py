@@ -1,9 +1,10 @@
-"""The automatic velocity-group count, from handles that are not bound (no GPU)."""
+"""The automatic velocity-group count, from handles that are not bound, and the default
+tile shape (no GPU)."""
 import ctypes
 
 import pytest
 
-from paper_2208_09132_gb300 import cdugks, workloads as wl
+from paper_2208_09132_gb300 import cdugks, tune, workloads as wl
 
 
 def automatic(cfg, prec, tile, recon=0):
@@ -58,3 +59,10 @@ def test_fp64_face_gradient_takes_at_least_four_waves(n, nv, groups):
     t = next(t for t in range(cdugks.load().cdugks_tile_count(cdugks.FP64, len(n)))
              if cdugks.tile_shape(cdugks.FP64, len(n), t)[1] & 8)
     assert automatic(cfg, cdugks.FP64, t, recon=1) == groups
+
+
+@pytest.mark.parametrize("n", [(3, 3), (10, 10), (11, 23), (16, 16), (40, 20), (256, 256)])
+def test_default_shape_of_2d_fp32_has_256_threads(n):
+    """Also on grids of fewer cells than any tile has."""
+    cfg, _ = wl.random_smooth(dim=2, n=n, nv=(9, 9), seed=1)
+    assert cdugks.tile_shape(cdugks.FP32, 2, tune.default_choice(cfg, cdugks.FP32)[0])[0] == (32, 8, 1)
