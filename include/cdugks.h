@@ -324,9 +324,11 @@ CDUGKS_API int cdugks_set_acceleration(cdugks_t *h, const double *a);
  * 0 restores normal operation).  While on, sweep A issues none of its tensor
  * copies and its wait gives up after 2^10 tries instead of 2^22: a step on a
  * tile shape that stages with tensor copies (the fused shapes of 1D/2D
- * problems large enough for interior tiles; those whose sweep A has upwind
- * owners run the staging sweep A while the hook is on) stops its sweep and the next
- * cdugks_sync_status reports CDUGKS_ERR_TIMEOUT.  Nothing faults or hangs;
+ * problems large enough for interior tiles) stops its sweep and the next
+ * cdugks_sync_status reports CDUGKS_ERR_TIMEOUT.  Of these the shapes without
+ * the face store and the face-gradient ones run that sweep A in every step; the
+ * other face-store shapes' own sweep A waits for nothing, and they run the
+ * staging one while the hook is on, and only then.  Nothing faults or hangs;
  * that step's results are incomplete (cdugks_init or cdugks_set_state
  * restores a valid state) and the handle stays usable.  Drops captured
  * graphs. */

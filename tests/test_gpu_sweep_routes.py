@@ -5,7 +5,7 @@ import pytest
 
 from paper_2208_09132_gb300 import cdugks, workloads as wl
 from test_gpu_parity import _bc
-from test_gpu_sweeps import check
+from test_gpu_sweeps import CASES, check
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +30,59 @@ def test_force_along_several_axes_on_rows_that_are_not_whole_chunks(oracle_mod, 
         s.init(f)
         s.step(3)
         check(s, o, prec, groups)
+
+
+STORED = [(prec, collision, case) for prec in (cdugks.FP32, cdugks.FP64) for collision in (0, 1) for case in CASES
+          if len(case[0]) == 3 or (len(case[0]) == 2 and prec == cdugks.FP32 and not collision)]
+STORED = [x for x in STORED if not any(DI in b for b in x[2][2])]      # (they take no Dirichlet ends)
+
+
+@pytest.mark.parametrize("prec,collision,case", STORED, ids=[
+    f"{'fp64' if p == cdugks.FP64 else 'fp32'}_{'shakhov_' if c else ''}{'x'.join(map(str, k[0]))}_nv{'x'.join(map(str, k[1]))}"
+    for p, c, k in STORED])
+def test_stored_face_store_at_tile_edges_matches_oracle(oracle_mod, prec, collision, case):
+    """Stored slopes and face store: sweep B with exchanged fluxes on its own tile,
+    in FP64 3D among them (the only face-store shapes of the default model there)."""
+    n, nv, bc = case
+    cfg, f = wl.random_smooth(dim=len(n), n=n, nv=nv, seed=sum(n) + nv[0], amp=0.2, kn=3e-3, vmax=5.0)
+    cfg = _bc(cfg, bc)
+    cfg["collision"] = collision
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(3)
+    checked = 0
+    for t in range(cdugks.load().cdugks_tile_count(prec, len(n))):
+        mode = cdugks.tile_shape(prec, len(n), t)[1]
+        if mode & ~16 != 6 or bool(mode & 16) != bool(collision):
+            continue
+        for groups in (1, 3, 64):
+            s = cdugks.Solver(cfg, precision=prec, tile_id=t, velocity_groups=groups)
+            s.init(f)
+            s.step(3)
+            check(s, o, prec, (t, groups))
+        checked += 1
+    assert checked >= 1
+
+
+@pytest.mark.parametrize("prec,D,cells,mode", [(cdugks.FP32, 1, (128,), 0), (cdugks.FP32, 2, (32, 8), 0), (cdugks.FP64, 1, (128,), 0),
+                                               (cdugks.FP64, 2, (8, 8), 12)])
+def test_wait_hook_on_sweeps_that_stage_in_production(oracle_mod, prec, D, cells, mode):
+    """The bounded wait of the sweeps that steps of these shapes run (the shapes with
+    upwind owners have no such wait and run the staging sweep under the hook only)."""
+    cfg, f = wl.random_smooth(dim=D, n=(1030,) if D == 1 else (72, 28), nv=(8, 8), seed=1, amp=0.3, kn=3e-3)
+    cfg["recon"] = 1 if mode & 8 else 0
+    lib = cdugks.load()
+    t = next(t for t in range(lib.cdugks_tile_count(prec, D))
+             if cdugks.tile_shape(prec, D, t) == (cells + (1,) * (3 - D), mode))
+    s = cdugks.Solver(cfg, precision=prec, tile_id=t)
+    s.init(f)
+    assert lib.cdugks_test_wait_timeout(s._h, 1) == 0
+    s.step(1)
+    assert s.sync_status() == cdugks.ERR_TIMEOUT
+    assert lib.cdugks_test_wait_timeout(s._h, 0) == 0
+    s.init(f)
+    s.step(3)
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(3)
+    check(s, o, prec, t)
