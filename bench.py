@@ -163,14 +163,15 @@ def measured_peak_hbm():
 
 def kernel_source_sha():
     """Hash of the sweep kernels' source (the section of kernels.cuh that holds
-    them, the lean sweeps, the persistent batched step and their launch
-    helpers): profile counters taken on other source are not reported."""
+    the staging sweeps, the sweeps with upwind owners and exchanged fluxes, the
+    factor tables, the persistent batched step and their launch helpers): profile
+    counters taken on other source are not reported."""
     csrc = os.path.join(ROOT, "paper_2208_09132_gb300", "csrc")
     txt = open(os.path.join(csrc, "kernels.cuh")).read()
     a = txt.index("// --------------------------------------------------------------- the sweep")
     b = txt.index("// Face constants from the group-summed face W")
     h = hashlib.sha256(txt[a:b].encode())
-    for f in ("lean.cuh", "persist.cuh", "sweeps_impl.cuh"):
+    for f in ("lean.cuh", "persist.cuh", "sweeps_impl.cuh", "pack.cuh", "usweep.cuh", "bflux.cuh"):
         h.update(open(os.path.join(csrc, f), "rb").read())
     return h.hexdigest()[:16]
 

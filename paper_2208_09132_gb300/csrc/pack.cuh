@@ -183,20 +183,6 @@ __device__ __forceinline__ Pk<double> ldg4(const double* p) {
     return {{a.x, a.y, b.x, b.y}};
 }
 
-// The same, loaded anew at each use (not kept in registers from one use to the next).
-__device__ __forceinline__ Pk<float> ldv4(const float* p) {
-    Pk<float> r;
-    asm volatile("ld.global.nc.v2.b64 {%0, %1}, [%2];" : "=l"(r.p[0]), "=l"(r.p[1]) : "l"(p));
-    return r;
-}
-__device__ __forceinline__ Pk<double> ldv4(const double* p) {
-    Pk<double> r;
-    asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];"
-                 : "=d"(r.v[0]), "=d"(r.v[1]), "=d"(r.v[2]), "=d"(r.v[3])
-                 : "l"(p));
-    return r;
-}
-
 // The van Leer limiter of the sweeps with upwind owners.  FP64: the quotient p / s
 // for p > 0 by residual correction with one FMA (P. Markstein, IBM J. Res. Dev. 34
 // (1990) 111): with an approximate reciprocal y of s and q = p y, twice

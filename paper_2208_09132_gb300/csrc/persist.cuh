@@ -129,10 +129,11 @@ __global__ void __launch_bounds__(Tile<D, TX, TY, TZ>::NT, (PersistSmem<T, D, TX
         }
         __syncthreads();
         if (!s_ok) break;
-        // Every body takes the member's record from the table directly: a copy
-        // of the whole record on every thread's stack, made again for every
-        // item, cost more than the items' own state traffic (each item's
-        // acquire also evicts the stack lines from L1, so they go out to L2).
+        // The sweeps read the member's record from shared memory, copied there once
+        // an item; the face and W items, which read it once or twice a thread, from
+        // the table.  (A copy on every thread's stack for every item cost more than
+        // the items' own state traffic: each item's acquire also evicts the stack
+        // lines from L1, so they go out to L2.)
         const int c = (cur[m] + s) & 1;
         const Inst<T>& in = insts[m];
         if (it.kind == PK_A) {

@@ -140,9 +140,9 @@ struct BLaunch {
     }
 };
 // The tile of sweep B (outside the persistent step, whose blocks are those of
-// the shape).  In FP32 CTAs of 128 threads: three per SM with up to 168
-// registers each (the chunk in flight, the next one's loads and the sums fit
-// without spills) overlap each other's barriers better than two of 256: 3D
+// the shape).  In FP32 CTAs of 128 threads: four per SM with up to 128 registers
+// each in 2D and in 3D with face tables, three with up to 168 in 3D without (shared
+// memory).  They overlap each other's barriers better than two of 256: 3D
 // 8 x 8 x 4 -> 8 x 4 x 4 12.0 -> 9.1 ps per point and step (32^3 x 24^3), 2D
 // 32 x 8 -> 32 x 4 5.94 -> 5.79 (256^2 x 32^2) and 7.98 -> 7.27 (100^2 x 101^2);
 // 16 x 8: 6.09 and 7.48.
