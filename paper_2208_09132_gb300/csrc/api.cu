@@ -381,7 +381,7 @@ void set_groups(cdugks* h, int G) {
         bool has[3][2] = {{false, false}, {false, false}, {false, false}};
         long long first = 0;                       // of the class
         for (int c = 0; c < 64; ++c) {
-            if (first < j1 && first + h->vcls[c] > j0)
+            if (h->vcls[c] && first < j1 && first + h->vcls[c] > j0)
                 for (int a = 0; a < g.D; ++a) {
                     has[a][cdg::visit_plus(c, a)] = true;
                     if (cdg::visit_mixed(c, a)) has[a][0] = true;

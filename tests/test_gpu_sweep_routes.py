@@ -4,6 +4,7 @@ import numpy as np
 import pytest
 
 from paper_2208_09132_gb300 import cdugks, workloads as wl
+from paper_2208_09132_gb300.tune import has_zero_node
 from test_gpu_parity import _bc
 from test_gpu_sweeps import CASES, check
 
@@ -86,3 +87,42 @@ def test_wait_hook_on_sweeps_that_stage_in_production(oracle_mod, prec, D, cells
     o.init(f)
     o.step(3)
     check(s, o, prec, t)
+
+
+# velocity ranges per axis: one sign only, a node at 0 at an end, uneven about 0
+RANGES = [((7,), [(0.1, 4.5)], [(P, P)], (11,)), ((32,), [(-4.5, -0.2)], [(DI, DI)], (70,)), ((9,), [(0.0, 4.0)], [(P, P)], (5,)),
+          ((7, 4), [(0.1, 4.5), (-4.5, 4.5)], [(P, P), (DI, DI)], (1, 2)), ((16, 9), [(-5.9, -0.2), (-5.9, 5.9)], [(P, P), (P, P)], (3, 19)),
+          ((8, 12), [(-3.8, 5.5), (-5.5, 5.5)], [(DI, DI), (S, DI)], (3, 8)), ((8, 5), [(-5.5, 3.3), (-5.5, 5.5)], [(DI, DI), (DI, S)], (12, 27)),
+          ((10, 13), [(-4.4, 4.4), (0.0, 4.4)], [(P, P), (DI, DI)], (1, 3)),
+          ((8, 8, 8), [(0.1, 5.5), (-5.5, 5.5), (-3.9, 5.5)], [(P, P), (S, S), (P, P)], (13, 2, 1)),
+          ((3, 8, 2), [(0.1, 4.8), (-4.8, -0.2), (-4.8, 4.8)], [(P, P), (P, P), (DI, DI)], (2, 11, 6)),
+          ((2, 8, 8), [(-3.8, 3.8), (-3.8, -0.2), (-3.8, 3.8)], [(DI, DI), (DI, DI), (S, S)], (3, 6, 2))]
+
+
+@pytest.mark.parametrize("prec", [cdugks.FP32, cdugks.FP64])
+@pytest.mark.parametrize("nv,ranges,bc,n", RANGES, ids=["x".join(map(str, r[0])) + "_n" + "x".join(map(str, r[3])) for r in RANGES])
+def test_velocity_ranges_of_one_sign_in_a_workspace_of_nans(oracle_mod, nv, ranges, bc, n, prec):
+    """Groups that lack a sign along an axis, alone and with others of several
+    classes: every partial sum and face value that is read has been written."""
+    import torch
+    D = len(nv)
+    cfg, f = wl.random_smooth(dim=D, n=n, nv=nv, seed=3, amp=0.1, kn=1e-2, vmax=4.0)
+    cfg = _bc(cfg, bc)
+    cfg["vlo"], cfg["vhi"] = [r[0] for r in ranges] + [-1.0] * (3 - D), [r[1] for r in ranges] + [1.0] * (3 - D)
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(2)
+    checked = 0
+    for t in range(cdugks.load().cdugks_tile_count(prec, D)):
+        mode = cdugks.tile_shape(prec, D, t)[1]
+        if not mode & 4 or mode & (8 | 16 | 32) or (mode & 128 and has_zero_node(cfg)) or (mode & 3 == 2 and DI in sum(bc, ())):
+            continue
+        checked += 1
+        for groups in (0, 1, 2, 3, 5, 6, 7, 64):
+            size = cdugks.Solver(cfg, precision=prec, tile_id=t, velocity_groups=groups).workspace_bytes
+            ws = torch.full((size + 256,), 255, dtype=torch.uint8, device="cuda:0")
+            s = cdugks.Solver(cfg, precision=prec, tile_id=t, velocity_groups=groups, workspace=ws)
+            s.init(f)
+            s.step(2)
+            check(s, o, prec, (t, groups))
+    assert checked or (D == 3 and prec == cdugks.FP64 and DI in sum(bc, ()))
