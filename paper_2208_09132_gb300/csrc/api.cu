@@ -711,9 +711,17 @@ int cdugks_create(const cdugks_grid* grid, const cdugks_vgrid* vgrid, const cdug
     consts(g.cd);
     // with Pr = 1 the TEDDF b-source coefficient (Pr - 1)/tau vanishes exactly
     g.nosrc = phys->Pr == 1.0;
+    // (a wall's ghost is an image of sweep A's upwind side only where mirrored nodes
+    // have opposite signs: the middle node of an odd grid may round to either one)
     g.mirror = 1;
     for (int a = 0; a < D; ++a)
-        for (int s = 0; s < 2; ++s) g.mirror = g.mirror && g.bc[a][s] != CDUGKS_BC_DIRICHLET;
+        for (int s = 0; s < 2; ++s) {
+            g.mirror = g.mirror && g.bc[a][s] != CDUGKS_BC_DIRICHLET;
+            for (int k = 0; k < nv[a] && g.bc[a][s] == CDUGKS_BC_SPECULAR; ++k) {
+                const double x = nodes[a][k], y = nodes[a][nv[a] - 1 - k];
+                g.mirror = g.mirror && (x > 0.0) == (y < 0.0) && (x < 0.0) == (y > 0.0);
+            }
+        }
     set_tiles(h, 0);
     h->vel32 = cast_vec<float>(h->vel);
     h->gsel = 0;

@@ -117,7 +117,8 @@ struct Geo {
     int upw;          // this instance's sweep A is usweep.cuh's
     int mixed;        // some visit is mixed along an axis
     int nvis;         // visits (chunk, sign pattern), in the order of Bufs::vint
-    int mirror;       // no Dirichlet end: ghosts are images of cells with all their neighbours
+    int mirror;       // no Dirichlet end, walls on grids that mirror sign to sign: ghosts are images of cells
+                      // with all their neighbours
     int ws[3];        // partial sums of the face W per axis: the group slots of sweep A (G where it sums both sides)
 };
 

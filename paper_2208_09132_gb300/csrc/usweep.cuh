@@ -31,8 +31,9 @@
 // value at xi is its cell's at the mirrored velocity, so the cell stores it
 // there as well, and the face moments are the cell's doubled, without the
 // normal momentum.  With a Dirichlet end (whose ghosts along one axis differ
-// from the images of their neighbours' ghosts) the end tiles form the ghosts'
-// values after the sweep (edge_pass).
+// from the images of their neighbours' ghosts), and between walls on a grid whose
+// middle node rounds to one side of 0 (it is its own image, of the same sign), the
+// end tiles form the ghosts' values after the sweep (edge_pass).
 //
 // What bounds it: in FP32 instruction issue and latency at 16 warps per SM, then the
 // 8 B read and 8 D B written per point; in FP64 the FP64 pipe.  Against left-face
@@ -296,8 +297,8 @@ __device__ __forceinline__ void store_lanes(T* dst, int lanes, const Pk<T>& vg, 
             dst[VC + v] = b4[v];
         }
 }
-// A cell at the ends `end` (1 low, 2 high) of axis a, on a grid without
-// Dirichlet ends: its face value (plus: of the right face; lanes st, of them zl
+// A cell at the ends `end` (1 low, 2 high) of axis a, on a grid of images
+// (Geo::mirror): its face value (plus: of the right face; lanes st, of them zl
 // at xi_a = 0) where a ghost beyond the end is its image.
 template <typename T>
 __device__ __forceinline__ void end_faces(const Geo& g, const Bufs<T>& bf, int a, int plus, int end, int vt, int st, int zl, int ff,

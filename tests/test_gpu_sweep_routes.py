@@ -126,3 +126,37 @@ def test_velocity_ranges_of_one_sign_in_a_workspace_of_nans(oracle_mod, nv, rang
             s.step(2)
             check(s, o, prec, (t, groups))
     assert checked or (D == 3 and prec == cdugks.FP64 and DI in sum(bc, ()))
+
+
+@pytest.mark.parametrize("prec", [cdugks.FP32, cdugks.FP64])
+@pytest.mark.parametrize("physics", ["plain", "shakhov", "force"])
+@pytest.mark.parametrize("D,axis,vmax,nodes", [(1, 0, 3.675, 7), (1, 0, 3.88, 7), (2, 0, 3.727, 11), (2, 1, 3.962, 11), (2, 1, 3.675, 7),
+                                               (2, 0, 5.964, 13), (3, 0, 3.88, 7), (3, 1, 3.675, 7), (3, 2, 3.88, 7)])
+def test_walls_on_odd_grids_whose_middle_node_rounds_off_zero(oracle_mod, D, axis, vmax, nodes, physics, prec):
+    """The middle node of -v .. v is 4e-16 or 9e-16 off 0 to either side: its mirror
+    image is itself, of the same sign, so a wall's ghost is not the image of the
+    cell's upwind side there."""
+    middle = -vmax + 2 * vmax * (nodes // 2) / (nodes - 1)
+    assert 0 < abs(middle) < 1e-15
+    nv = [8, 6, 4][:D]
+    nv[axis] = nodes
+    cfg, f = wl.random_smooth(dim=D, n=(19, 11, 6), nv=nv, seed=9, amp=0.1, kn=3e-3, vmax=vmax)
+    cfg = _bc(cfg, [(S, S) if a == axis else (P, P) for a in range(D)])
+    cfg["collision"] = 1 if physics == "shakhov" else 0
+    if physics == "force":
+        cfg["accel"] = [0.2 if a == axis else -0.1 for a in range(D)] + [0.0] * (3 - D)
+    o = oracle_mod.Oracle(cfg)
+    o.init(f)
+    o.step(3)
+    checked = 0
+    for t in range(cdugks.load().cdugks_tile_count(prec, D)):
+        mode = cdugks.tile_shape(prec, D, t)[1]
+        if not mode & 4 or mode & 8 or bool(mode & 16) != (physics == "shakhov") or bool(mode & 32) != (physics == "force"):
+            continue
+        checked += 1
+        for groups in (0, 1, 5):
+            s = cdugks.Solver(cfg, precision=prec, tile_id=t, velocity_groups=groups)
+            s.init(f)
+            s.step(3)
+            check(s, o, prec, (t, groups))
+    assert checked
