@@ -802,8 +802,10 @@ int cdugks_set_tile(cdugks_t* h, int tile_id) {
         }
         set_groups(h, G);
     }
-    if (h->bound) return upload_inst(h);
-    return CDUGKS_OK;
+    if (!h->bound) return CDUGKS_OK;
+    const cudaError_t e = h->prec == CDUGKS_FP32 ? cdg::prepare_shape_f32(h->g.D, tile_id) : cdg::prepare_shape_f64(h->g.D, tile_id);
+    if (e) return cuda_fail(e, "load the sweeps");
+    return upload_inst(h);
 }
 
 int cdugks_workspace_bytes(const cdugks_t* h, size_t* bytes) {
@@ -942,7 +944,8 @@ int cdugks_bind(cdugks_t* h, void* device_ptr, size_t bytes, void* cuda_stream) 
     }
     if ((e = cudaMemsetAsync(h->base + h->lay.status, 0, 256, h->stream))) return cuda_fail(e, "clear status");
     if ((e = cudaStreamSynchronize(h->stream))) return cuda_fail(e, "cudaStreamSynchronize");
-    (void)g;
+    if ((e = f32 ? cdg::prepare_shape_f32(g.D, g.tile_id) : cdg::prepare_shape_f64(g.D, g.tile_id)))
+        return cuda_fail(e, "load the sweeps");
     h->bound = true;
     h->initialised = false;
     return upload_inst(h);

@@ -47,6 +47,10 @@ int sweep_a_ctas_f32(int D, int id);              // CTAs of sweep A per SM
 int sweep_a_ctas_f64(int D, int id);
 int sweep_b_ctas_f32(int D, int id);              // of sweep B
 int sweep_b_ctas_f64(int D, int id);
+// Loads and configures the sweeps of a shape (otherwise the first step does: 10 to 18
+// ms for the first of a precision and dimension in a process).
+cudaError_t prepare_shape_f32(int D, int id);
+cudaError_t prepare_shape_f64(int D, int id);
 size_t sweep_smem_f32(int D, int id);
 size_t sweep_smem_f64(int D, int id);
 // Sweep mode of a shape (MODE_FUSED / MODE_PREP / MODE_STORED): prepared and

@@ -9,6 +9,7 @@ TileShape tile_shape_f32(int D, int id) { return shapes_of<float>(D).shape(id); 
 TileShape b_tile_shape_f32(int D, int id) { return shapes_of<float>(D).b_shape(id); }
 int sweep_a_ctas_f32(int D, int id) { return shapes_of<float>(D).a_ctas(id); }
 int sweep_b_ctas_f32(int D, int id) { return shapes_of<float>(D).b_ctas(id); }
+cudaError_t prepare_shape_f32(int D, int id) { return shapes_of<float>(D).configure(id); }
 size_t sweep_smem_f32(int D, int id) { return shapes_of<float>(D).smem(id); }
 int tile_mode_f32(int D, int id) { return shapes_of<float>(D).mode(id); }
 

@@ -10,6 +10,7 @@ TileShape tile_shape_f64(int D, int id) { return shapes_of<double>(D).shape(id);
 TileShape b_tile_shape_f64(int D, int id) { return shapes_of<double>(D).b_shape(id); }
 int sweep_a_ctas_f64(int D, int id) { return shapes_of<double>(D).a_ctas(id); }
 int sweep_b_ctas_f64(int D, int id) { return shapes_of<double>(D).b_ctas(id); }
+cudaError_t prepare_shape_f64(int D, int id) { return shapes_of<double>(D).configure(id); }
 size_t sweep_smem_f64(int D, int id) { return shapes_of<double>(D).smem(id); }
 int tile_mode_f64(int D, int id) { return shapes_of<double>(D).mode(id); }
 

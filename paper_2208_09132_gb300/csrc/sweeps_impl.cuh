@@ -503,6 +503,7 @@ struct ShapeList<> {
     static TileShape b_shape(int) { return {{0, 0, 0}}; }
     static int a_ctas(int) { return 1; }
     static int b_ctas(int) { return 1; }
+    static cudaError_t configure(int) { return cudaErrorInvalidValue; }
     static size_t smem(int) { return 0; }
     static int mode(int) { return 0; }
     static bool persistent(int) { return false; }
@@ -532,6 +533,7 @@ struct ShapeList<H, R...> {
     static TileShape b_shape(int id) { return id == 0 ? H::b_shape() : Rest::b_shape(id - 1); }
     static int a_ctas(int id) { return id == 0 ? H::a_ctas() : Rest::a_ctas(id - 1); }
     static int b_ctas(int id) { return id == 0 ? H::b_ctas() : Rest::b_ctas(id - 1); }
+    static cudaError_t configure(int id) { return id == 0 ? H::configure() : Rest::configure(id - 1); }
     static size_t smem(int id) { return id == 0 ? H::smem_bytes() : Rest::smem(id - 1); }
     static int mode(int id) { return id == 0 ? H::mode : Rest::mode(id - 1); }
     static bool persistent(int id) { return id == 0 ? H::persistent : Rest::persistent(id - 1); }
@@ -553,6 +555,7 @@ struct ShapeOps {
     TileShape (*b_shape)(int);      // the tile of sweep B's batched items
     int (*a_ctas)(int);             // CTAs of sweep A per SM
     int (*b_ctas)(int);             // of sweep B
+    cudaError_t (*configure)(int);
     size_t (*smem)(int);
     int (*mode)(int);
     bool (*persistent)(int);
@@ -562,7 +565,7 @@ struct ShapeOps {
 };
 template <typename T, typename L>
 ShapeOps<T> ops_of() {
-    return {L::count, &L::shape, &L::b_shape, &L::a_ctas, &L::b_ctas, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
+    return {L::count, &L::shape, &L::b_shape, &L::a_ctas, &L::b_ctas, &L::configure, &L::smem, &L::mode, &L::persistent, &L::template step<T>,
             &L::template sweep_batch<T>, &L::template persist<T>};
 }
 const ShapeOps<float>& shapes_f32_1();
